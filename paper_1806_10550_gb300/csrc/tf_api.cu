@@ -333,6 +333,60 @@ std::mutex g_tune_mutex;
 std::vector<std::pair<TuneKey, int>> g_tune;
 TuneKey tune_key(const tf_params& p) { return TuneKey{p.nx, p.ny, p.precision, p.model, p.n, p.m}; }
 
+// Lines per block of a sweep over n lines.  A line's recurrence is a chain, so
+// a block's tick hardly shortens with fewer lines, but a film whose blocks of
+// 32 lines leave SMs idle runs in fewer lines per SM when each smaller block
+// still has an SM of its own, or, in FP32-bulk, half of one.  Measured, us per x
+// / y sweep at 4, 8, 16 and 32 lines a block: FP32-bulk 512^2 22/27, 23/29, 27/35,
+// 38/45; 1024^2 39/47, 37/45, 45/57, 69/81; 2048^2 129/144, 74/90, 79/100, 130/154;
+// 4096^2 at 8, 16 and 32 lines 267/326, 182/235, 254/305; 8192^2 at 16 and 32
+// 627/791, 734/802.  With the out-of-line mobilities (NLC) the producers are
+// the longest role, and 4 lines win further: 1024^2 86/89, 115/121, 134/143;
+// 2048^2 309/322, 227/241, 255/270; 4096^2 at 8 and 16 lines 875/928, 644/665.
+// FP64 512^2 164/166, 170/174, 202/211, 331/351; 1024^2 377/615, 317/322, 379/391,
+// 647/687; 2048^2 at 8, 16 and 32 lines 1197/1221, 732/752, 1278/1348; from there
+// on one block an SM, and blocks of 32 do less work per line.
+constexpr int kSMs = 152;
+int sweep_lines(int n, int precision, bool general) {
+  if (n <= 4 * kSMs * (precision != TF_FP64 && general ? 2 : 1)) return 4;
+  if (n <= 8 * kSMs * (precision != TF_FP64 ? 2 : 1)) return 8;
+  return precision != TF_FP64 || n <= 16 * kSMs ? 16 : 32;
+}
+// Fewest lines per block for films that run at once, by the sum of their line
+// counts: smaller blocks do more work per line, which only pays while the
+// films together leave SMs idle.  Whole runs in FP32-bulk, us at 8, 16 and 32
+// lines: 15 films of 4630 lines in all 1179, 1169, 1260; 11 of 7968 4365, 3536,
+// 3618; 23 of 10686 4583, 3787, 3936; 24 of 15365 7107, 5738, 5391.
+int shared_lines(long long lines) {
+  return lines <= 8 * kSMs ? 4 : (lines <= 16 * kSMs ? 8 : (lines <= 80 * kSMs ? 16 : 32));
+}
+// The sweeps' block shape, at least `least` lines per block.  In FP32-bulk with
+// the out-of-line mobility models the shapes round differently, so there the
+// shape depends on the film alone.
+void set_lines(tf_ctx& c, int least) {
+  if (c.p.precision != TF_FP64 && !c.packed_rhs) least = 0;
+  const bool general = !(c.mk.model == TF_MODEL_POWERLAW && c.mk.n == 3 && c.mk.m == 2);
+  const int x = sweep_lines(c.p.ny, c.p.precision, general), y = sweep_lines(c.p.nx, c.p.precision, general);
+  c.nlx = x > least ? x : least;
+  c.nly = y > least ? y : least;
+  c.grid_x = (c.p.ny + c.nlx - 1) / c.nlx;
+  c.grid_y = (c.p.nx + c.nly - 1) / c.nly;
+}
+// Films that advance at once run in blocks of at least shared_lines() lines;
+// their contexts go back to the shapes of a film alone afterwards.
+struct SharedLines {
+  int n;
+  tf_ctx* const* ctx;
+  SharedLines(int n_, tf_ctx* const* c) : n(n_), ctx(c) {
+    long long lines = 0;
+    for (int i = 0; i < n; ++i) lines += ctx[i]->p.nx > ctx[i]->p.ny ? ctx[i]->p.nx : ctx[i]->p.ny;
+    for (int i = 0; i < n; ++i) set_lines(*ctx[i], shared_lines(lines));
+  }
+  ~SharedLines() {
+    for (int i = 0; i < n; ++i) set_lines(*ctx[i], 0);
+  }
+};
+
 template <class T> int dalloc(T** p, size_t bytes) {
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, bytes ? bytes : 16);
@@ -509,8 +563,6 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
   mk.pol_A1 = p->pol_A_SiOx;
   mk.pol_A2 = p->pol_A_Si;
   mk.pol_d = p->pol_d;
-  c->grid_x = (p->ny + 31) / 32;
-  c->grid_y = (p->nx + 31) / 32;
   c->grid_rx = (p->nx + 31) / 32;
   c->grid_ry = (p->ny + 31) / 32;
   {
@@ -525,6 +577,7 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
     c->grid_pkx = (int)((warps + tf::kRhsStripWarps - 1) / tf::kRhsStripWarps);
   }
   c->packed_rhs = p->precision != TF_FP64 && p->model == TF_MODEL_POWERLAW && p->n == 3 && p->m == 2;
+  set_lines(*c, 0);
   c->n_rhs_parts = c->packed_rhs ? c->grid_pkx : c->grid_rx * c->grid_ry;
   c->grid_st_x = (p->nx + 15) / 16;
   c->grid_st_y = (p->ny + 15) / 16;
@@ -535,9 +588,10 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
   }
   c->n_py = c->grid_y > c->grid_stats ? c->grid_y : c->grid_stats;
   const size_t hp = c->ops->hp_bytes, lp = c->ops->lp_bytes;
-  // factor scratch: one slab per block of 32 lines, line half and chunk
-  const size_t facx = tf::fac_slab<tf::kCX>(c->grid_x, 0, 0, tf::chunks_per_half<tf::kCX>(p->nx));
-  const size_t facy = tf::fac_slab<tf::kRY>(c->grid_y, 0, 0, tf::chunks_per_half<tf::kRY>(p->ny));
+  // factor scratch: one slab per sweep block, line half and chunk
+  // (sized for blocks of 32, the most that a partly filled last block takes)
+  const size_t facx = tf::fac_slab<tf::kCX>(32, (p->ny + 31) / 32, 0, 0, tf::chunks_per_half<tf::kCX>(p->nx));
+  const size_t facy = tf::fac_slab<tf::kRY>(32, (p->nx + 31) / 32, 0, 0, tf::chunks_per_half<tf::kRY>(p->ny));
   int r = TF_OK;
   cudaError_t e = c->ops->prepare();
   if (e != cudaSuccess) r = cuda_fail(e);
@@ -717,6 +771,10 @@ int tf_advance(tf_ctx* c, double* h, double t0, double t_end, double dt0, int ma
 bool graph_capable(const tf_ctx& c) { return c.ops->ens_graph && c.packed_rhs && !c.part; }
 
 int film_graph_start(tf_ctx& c, double* h, double t0, double t_end, double dt0, int max_att, int streak) {
+  if (c.ens_exec && (c.ens_nlx != c.nlx || c.ens_nly != c.nly)) {  // built for other block shapes
+    TF_CK(cudaGraphExecDestroy(c.ens_exec));
+    c.ens_exec = nullptr;
+  }
   if (!c.ens_exec) {  // first use; a failed earlier build keeps its buffers
     if (!c.ens_dev) {
       int r = dalloc((void**)&c.ens_dev, sizeof(tf::EnsDev));
@@ -724,6 +782,8 @@ int film_graph_start(tf_ctx& c, double* h, double t0, double t_end, double dt0, 
     }
     if (!c.ens_host) TF_CK(cudaMallocHost((void**)&c.ens_host, sizeof(tf::EnsDev)));
     TF_CK(c.ops->ens_graph(c, c.ens_dev, &c.ens_exec));
+    c.ens_nlx = c.nlx;
+    c.ens_nly = c.nly;
   }
   tf::EnsDev& e = *c.ens_host;
   memset(&e, 0, sizeof(e));
@@ -788,6 +848,7 @@ int tf_ensemble_advance(int n, tf_ctx* const* ctx, double* const* h, const doubl
     for (int j = 0; j < i; ++j)
       if (ctx[j] == ctx[i]) return TF_ERR_ARG;  // one context per film
   }
+  const SharedLines shapes(n, ctx);
   // films on the graph engine: launched first, collected at the end
   std::vector<char> on_graph((size_t)n, 0);
   for (int i = 0; i < n; ++i) {
@@ -906,6 +967,7 @@ int tf_tune_line_solver(const tf_params* p, void* stream, const double* h, doubl
         break;
       }
       rc = tf_init(&q, st[(size_t)k], &ctx[(size_t)k]);
+      if (!rc) set_lines(*ctx[(size_t)k], shared_lines((long long)copies * (q.nx > q.ny ? q.nx : q.ny)));
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!rc && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) rc = TF_ERR_CUDA;

@@ -6,7 +6,7 @@
 #include <stddef.h>
 
 #include "../../include/tf.h"
-#include "tf_line_sweeps.cuh"
+#include "tf_narrow_sweeps.cuh"
 
 namespace tf {
 
@@ -87,8 +87,9 @@ struct tf_ctx {
   const tf::Ops* ops;
   cudaStream_t stream;
   size_t N;
-  int grid_x;      // blocks of the x sweep (32 rows each)
-  int grid_y;      // blocks of the y sweep (32 columns each)
+  int nlx, nly;    // lines per block of the x and y sweeps
+  int grid_x;      // blocks of the x sweep (nlx rows each)
+  int grid_y;      // blocks of the y sweep (nly columns each)
   int grid_rx, grid_ry;      // 2-D residual grid (32 x 32 tiles)
   int grid_pkx;              // packed FP32-bulk residual: blocks of kRhsStripWarps strip segments
   int strip_n, strip_rows;   // its strips across x and rows per segment
@@ -126,4 +127,5 @@ struct tf_ctx {
   tf::EnsDev* ens_dev;        // the film's device-resident controller state
   tf::EnsDev* ens_host;       // pinned staging copy of it
   cudaGraphExec_t ens_exec;   // the instantiated graph of a whole run
+  int ens_nlx, ens_nly;       // the lines per sweep block it was built with
 };

@@ -559,6 +559,28 @@ __device__ __forceinline__ void face_dF(const CellLP<LP>& P, const CellLP<LP>& Q
   dF[3] = wq * c3;
 }
 
+// Reciprocal of the FP64 line solves and of the FP64 Jacobian's heights: a
+// float seed r0 of 1/x (relative error e = 1 - x r0 of about 2^-22, the
+// mantissas crossing between the formats with integer operations) and one
+// third-order step, 1/x = r0 (1 + e + e^2) + O(e^3): three FP64 operations,
+// rounded once at the end.  What bounds the FP64 sweeps is the number of FP64
+// instructions (a warp's takes 64 cycles of its sub-partition's pipe whatever
+// its lanes).  Zero, non-finite and extreme arguments take the division.
+__device__ __forceinline__ double rcp3(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ex = (hi >> 20) & 0x7ffu;
+  if (ex - 64u > 1918u) return 1.0 / x;  // the seed and 1/x are normal for exponents 64 .. 1982
+  const float m = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));  // |x| / 2^(ex - 1023), truncated
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(m));  // in [1/2, 1]
+  const unsigned rb = __float_as_uint(r);
+  const double r0 =
+      __hiloint2double((int)(((rb >> 3) + ((896u + 1023u - ex) << 20)) | (hi & 0x80000000u)), (int)(rb << 29));
+  const double e = fma(-x, r0, 1.0);
+  return fma(r0, fma(e, e, e), r0);
+}
+__device__ __forceinline__ float rcp3(float x) { return rcp(x); }
+
 template <class LP> struct LUState {
   LP g1, d1, z1, g2, d2, z2;  // (gamma, delta, z) of rows i-1 and i-2
   __device__ __forceinline__ void reset() { g1 = d1 = z1 = g2 = d2 = z2 = LP(0); }
@@ -568,7 +590,7 @@ template <class LP> struct LUState {
   __device__ __forceinline__ void step(LP a, LP b, LP c, LP d, LP e, LP r, LP& g, LP& dl, LP& z, LP& chk) {
     LP beta = b - a * g2;
     LP mu = c - a * d2 - beta * g1;
-    LP inv = rcp(mu);
+    LP inv = rcp3(mu);
     g = (d - beta * d1) * inv;
     dl = e * inv;
     z = (r - a * z2 - beta * z1) * inv;
@@ -595,7 +617,7 @@ __device__ __forceinline__ void band_row(const LP L[4], const LP R[4], LP& a, LP
 // ---------------------------------------------------------------------------
 // per-cell helpers of the update and the Newton test
 
-__device__ __forceinline__ double rel_update(double v, double uk) { return fabs(v / uk); }
+__device__ __forceinline__ double rel_update(double v, double uk) { return fabs(v * rcp3(uk)); }
 __device__ __forceinline__ float rel_update(float v, double uk) {
   return __fdividef(fabsf(v), f32_of_pos_f64_fast(uk));  // uk > 0 or the step fails anyway
 }

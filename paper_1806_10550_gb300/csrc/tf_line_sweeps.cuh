@@ -1,4 +1,5 @@
-// tf_line_sweeps.cuh -- warp-specialised line sweeps.
+// tf_line_sweeps.cuh -- warp-specialised line sweeps in blocks of 32 lines (see
+// tf_narrow_sweeps.cuh for blocks of fewer lines).
 //
 // The exact twisted LU solve of every line (see tf_sweeps.cuh) has a short
 // sequential recurrence per cell; everything else per cell (the film values,
@@ -117,19 +118,20 @@ __device__ __forceinline__ void copy_rows(T* dst, const T* __restrict__ src, int
   }
 }
 
-// n <= NMAX contiguous elements; 16-byte vectors when both ends are aligned.
-template <class T, int NMAX>
+// n <= NMAX contiguous elements by NTH threads; 16-byte vectors when both ends
+// are aligned.
+template <int NTH, class T, int NMAX>
 __device__ __forceinline__ void copy_span(T* dst, const T* __restrict__ src, int n, int p) {
-  constexpr int V = 16 / sizeof(T), NI = (NMAX / V + kNP - 1) / kNP;
+  constexpr int V = 16 / sizeof(T), NI = (NMAX / V + NTH - 1) / NTH;
   if ((n % V) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
-      const int k = p + i * kNP;
+      const int k = p + i * NTH;
       if (k < n / V) __pipeline_memcpy_async(dst + k * V, src + k * V, 16);
     }
   } else {
 #pragma unroll 1
-    for (int k = p; k < n; k += kNP) cpT(dst + k, src + k);
+    for (int k = p; k < n; k += NTH) cpT(dst + k, src + k);
   }
 }
 
@@ -154,13 +156,13 @@ template <class LP> struct CellS {
   LP u, lap, F0, F1, D0, D1;
 };
 
-template <class LP, class Acc>
-__device__ __forceinline__ CellS<LP> cell_scaled(const MobC<LP>& ml, LP inv_ds2, LP k3, LP k1, Acc U) {
+// uc: the cell's height; lap: its unscaled Laplacian.
+template <class LP>
+__device__ __forceinline__ CellS<LP> cell_scaled(const MobC<LP>& ml, LP inv_ds2, LP k3, LP k1, LP uc, LP lap) {
   CellS<LP> X;
-  const LP uc = U(0, 0);
   X.u = uc;
-  X.lap = (((U(0, 1) - uc) + (U(0, -1) - uc)) + ((U(1, 0) - uc) + (U(-1, 0) - uc))) * inv_ds2;
-  const LP s = rcp(uc);
+  X.lap = lap * inv_ds2;
+  const LP s = rcp3(uc);
   LP f0, f1, d0, d1;
   mobility_all(ml, uc, s, f0, f1, d0, d1);
   X.F0 = k3 * f0;
@@ -173,13 +175,12 @@ __device__ __forceinline__ CellS<LP> cell_scaled(const MobC<LP>& ml, LP inv_ds2,
 // The same values for the (n, m) = (3, 2) power law with the constant
 // factors folded on the host (LineK): the Laplacian is left unscaled and
 // 1/ds^2 moves into D0, so faces see the same products.
-template <class LP, class Acc>
-__device__ __forceinline__ CellS<LP> cell_pl32(const LineK<LP>& L, Acc U) {
+template <class LP>
+__device__ __forceinline__ CellS<LP> cell_pl32(const LineK<LP>& L, LP uc, LP lap) {
   CellS<LP> X;
-  const LP uc = U(0, 0);
   X.u = uc;
-  X.lap = ((U(0, 1) - uc) + (U(0, -1) - uc)) + ((U(1, 0) - uc) + (U(-1, 0) - uc));
-  const LP s = rcp(uc), h2 = uc * uc;
+  X.lap = lap;
+  const LP s = rcp3(uc), h2 = uc * uc;
   // F0 rounded as a product of its own (never fused into the face sums
   // F0_p + F0_q) and F1 as one written-out fma: every instantiation of the
   // sweeps then rounds the band alike
@@ -190,10 +191,11 @@ __device__ __forceinline__ CellS<LP> cell_pl32(const LineK<LP>& L, Acc U) {
   return X;
 }
 
+// du = u_q - u_p
 template <class LP>
-__device__ __forceinline__ void face_scaled(const CellS<LP>& P, const CellS<LP>& Q, bool pl, bool qr,
+__device__ __forceinline__ void face_scaled(const CellS<LP>& P, const CellS<LP>& Q, LP du, bool pl, bool qr,
                                             LP dF[4]) {
-  const LP dl = Q.lap - P.lap, du = Q.u - P.u;
+  const LP dl = Q.lap - P.lap;
   const LP c3 = P.F0 + Q.F0, Bd = P.F1 + Q.F1;
   // one fused form, written out, so that every instantiation of the sweeps
   // rounds these alike (a * b + c * d may otherwise fuse either product)
@@ -216,33 +218,44 @@ __device__ __forceinline__ void face_scaled(const CellS<LP>& P, const CellS<LP>&
 // registers straight from the staged film tile: the scaled film values of the
 // G + 2 cells ia-1 .. ia+G, the G + 1 faces between them, and each row from
 // the derivatives of its two face fluxes (a..e multiply x_{i-2}..x_{i+2}).
-// A(s, dr, dc) is the film at line cell ia + s offset by (dr, dc) in the grid.
+// A(s, dr, dc) is the film at line cell ia + s offset by (dr, dc) in the grid;
+// DIR 0: the line runs along the grid's rows (dc), 1: along its columns (dr).
+// The differences of neighbours along the line serve both the Laplacians and
+// the faces.
 // EDGE: the group may reach a wall, where the outer face of an end cell
 // vanishes and faces next to a wall lose their outer stencil weight; without
 // EDGE (ia >= 2 and ia + G + 1 < n) every face is interior.  PL32 selects
 // the folded (n, m) = (3, 2) power law.  OUT(s, a, b, c, d, e) receives the
 // row of cell ia + s.
-template <class LP, int G, bool EDGE, bool PL32, class Acc, class Out>
+template <class LP, int G, int DIR, bool EDGE, bool PL32, class Acc, class Out>
 __device__ __forceinline__ void band_rows(const LineK<LP>& L, Acc A, int ia, int ib, int n, Out out) {
   CellS<LP> C[G + 2];
+  LP u[G + 4], du[G + 3];  // cells ia-2 .. ia+G+1 of the line and their differences
+#pragma unroll
+  for (int s = 0; s < G + 4; ++s) u[s] = A(s - 2, 0, 0);
+#pragma unroll
+  for (int s = 0; s < G + 3; ++s) du[s] = u[s + 1] - u[s];
 #pragma unroll
   for (int s = -1; s <= G; ++s) {
-    auto U = [&](int dr, int dc) { return A(s, dr, dc); };
+    const LP uc = u[s + 2];
+    const LP a = A(s, DIR == 0 ? 1 : 0, DIR == 0 ? 0 : 1) - uc, b = A(s, DIR == 0 ? -1 : 0, DIR == 0 ? 0 : -1) - uc;
+    // (right - u) + (left - u) along x, then along y
+    const LP lap = DIR == 0 ? (du[s + 2] - du[s + 1]) + (a + b) : (a + b) + (du[s + 2] - du[s + 1]);
     if constexpr (PL32)
-      C[s + 1] = cell_pl32<LP>(L, U);
+      C[s + 1] = cell_pl32<LP>(L, uc, lap);
     else
-      C[s + 1] = cell_scaled<LP>(L.ml, L.inv_ds2, L.k3, L.k1, U);
+      C[s + 1] = cell_scaled<LP>(L.ml, L.inv_ds2, L.k3, L.k1, uc, lap);
   }
   LP F[G + 1][4];
 #pragma unroll
   for (int f = 0; f <= G; ++f) {  // face between cells ia + f - 1 and ia + f
     if (EDGE) {
       const int q = ia + f - 1;
-      face_scaled(C[f], C[f + 1], q > 0, q + 2 < n, F[f]);
+      face_scaled(C[f], C[f + 1], du[f + 1], q > 0, q + 2 < n, F[f]);
       if (!(q >= 0 && q + 1 < n))
         for (int k = 0; k < 4; ++k) F[f][k] = LP(0);
     } else {
-      face_scaled(C[f], C[f + 1], true, true, F[f]);
+      face_scaled(C[f], C[f + 1], du[f + 1], true, true, F[f]);
     }
   }
 #pragma unroll
@@ -281,40 +294,41 @@ __device__ __forceinline__ void lu_chunk(LUState<LP>& lu, const LP* B, int lane,
   if (!(chk == chk)) bad = 1;
 }
 
-// Factor scratch of a sweep: for every block of 32 lines, line half and
-// chunk, one slab [g, d, z][cell][line] of 3 * L * 32 values, cells in the
+// Factor scratch of a sweep: for every block of nl lines, line half and
+// chunk, one slab [g, d, z][cell][line] of 3 * L * nl values, cells in the
 // solver's processing order; the backward pass stages a slab with one
 // contiguous copy.
 template <int L> __host__ __device__ inline int chunks_per_half(int n) {
-  const int m = split_point<L>(n);
+  const int m = split_point(n);
   const int a = (m + L - 1) / L, b = m < n ? (n - m + L - 1) / L : 0;
   return a > b ? a : b;
 }
-template <int L> __host__ __device__ inline size_t fac_slab(int blk, int h, int q, int nch) {
-  return (((size_t)blk * 2 + h) * nch + q) * (size_t)(3 * L * 32);
+template <int L> __host__ __device__ inline size_t fac_slab(int nl, int blk, int h, int q, int nch) {
+  return (((size_t)blk * 2 + h) * nch + q) * (size_t)(3 * L * nl);
 }
 
 // Back substitution x = z - g x' - d x'' over the n cells of one chunk in
 // processing order s = 0..n-1 (outward from the seam).  F(f, s) reads factor
-// f (g, d, z) of cell s; cells with IS_SEAM(s) take the seam solution XS(s);
-// PUT(s, x) stores x.  Chunks without seam cells run unrolled.
-template <class LP, int L, class Fac, class SeamF, class XsF, class Put>
-__device__ __forceinline__ void bs_chunk(LP& x1, LP& x2, int n, bool any_seam, Fac F, SeamF is_seam,
-                                         XsF xs, Put put) {
-  auto one = [&](int s, bool chk) {
-    const LP x = (chk && is_seam(s)) ? xs(s) : F(2, s) - F(0, s) * x1 - F(1, s) * x2;
+// f (g, d, z) of cell s; PUT(s, x) stores x.  The cells at the seam are no
+// exception: the recurrence starts from the two unknowns beyond them and
+// their rows are rows of the seam's system.  The newest value enters last, so
+// that the chain is one operation a cell: at 1024^2 (8 lines a block) a
+// 24-cell chunk of the FP32 x sweep went from 1250 to 650 cycles, of the FP64
+// one from 5070 to 4230.
+template <class LP, int L, class Fac, class Put>
+__device__ __forceinline__ void bs_chunk(LP& x1, LP& x2, int n, Fac F, Put put) {
+  auto one = [&](int s) {
+    const LP x = fma(-F(0, s), x1, fma(-F(1, s), x2, F(2, s)));
     x2 = x1;
     x1 = x;
     put(s, x);
   };
-  if (!any_seam && n == L) {
+  if (n == L) {
 #pragma unroll
-    for (int s = 0; s < L; ++s) one(s, false);
-  } else if (!any_seam) {
-#pragma unroll 8
-    for (int s = 0; s < n; ++s) one(s, false);
+    for (int s = 0; s < L; ++s) one(s);
   } else {
-    for (int s = 0; s < n; ++s) one(s, true);
+#pragma unroll 8
+    for (int s = 0; s < n; ++s) one(s);
   }
 }
 
@@ -347,7 +361,11 @@ template <class LP> struct YSmem {
 
 // DEV (the ensemble graphs): the step's band constants *Ld and the
 // iterates {u_k, u_k+1} = uio[0], uio[1] come from device memory.
-template <class Mode, bool DEV = false>
+// GEN: the mobility models other than the (3, 2) power law.  Kernels of their
+// own: their out-of-line calls cost the power law's kernels registers (the
+// ensemble graphs' sweeps spilled 230 bytes a thread and a 24-film run took
+// 6.0 ms against 5.4).
+template <class Mode, bool DEV, bool GEN>
 __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
     k_ysweep(ModelK M, LineK<typename Mode::LP> Lp, const double* __restrict__ up,
              const typename Mode::LP* __restrict__ ul, const typename Mode::LP* __restrict__ w,
@@ -365,7 +383,7 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
   const int p = threadIdx.x - 64;  // producer index (valid when !solver)
   const int nx = M.nx, ny = M.ny;
   const int i0 = blockIdx.x * 32;
-  const int m = split_point<kRY>(ny);
+  const int m = split_point(ny);
   const bool twisted = m < ny;
   // chunks per half (a runtime-indexed array would live in local memory)
   const int nch0 = (m + kRY - 1) / kRY, nch1 = twisted ? (ny - m + kRY - 1) / kRY : 0;
@@ -428,12 +446,12 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
                 q[5 * kRY * 32] = W[s * 32];
               };
               const bool edge = !(ja >= 2 && ja + kG + 1 < ny);
-              if (!L.ml.pl32)  // general exponents or the linear model
-                band_rows<LP, kG, true, false>(L, A, ja, jb, ny, out);
+              if (GEN)  // other exponents and models
+                band_rows<LP, kG, 1, true, false>(L, A, ja, jb, ny, out);
               else if (!edge)
-                band_rows<LP, kG, false, true>(L, A, ja, jb, ny, out);
+                band_rows<LP, kG, 1, false, true>(L, A, ja, jb, ny, out);
               else
-                band_rows<LP, kG, true, true>(L, A, ja, jb, ny, out);
+                band_rows<LP, kG, 1, true, true>(L, A, ja, jb, ny, out);
             }
           }
         }
@@ -443,7 +461,7 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
       if (q < nchh(h) && i0 + lane < nx) {
         const int r0 = r0_of(h, q), r1 = r1_of(h, q);
         const LP* B = &S.s.f.band[q & 1][h][0][0][0];
-        lu_chunk<LP, kRY>(lu, B, lane, r1 - r0, fac + fac_slab<kRY>(blockIdx.x, h, q, nch) + lane, pivot_bad);
+        lu_chunk<LP, kRY>(lu, B, lane, r1 - r0, fac + fac_slab<kRY>(32, blockIdx.x, h, q, nch) + lane, pivot_bad);
       }
     }
     __syncthreads();
@@ -467,7 +485,7 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
     for (int h = 0; h < 2; ++h) {
       const int q = nchh(h) - 1 - bq;
       if (q < 0) continue;
-      copy_span<LP, 3 * kRY * 32>(&S.s.b.ft[slot][h][0][0][0], fac + fac_slab<kRY>(blockIdx.x, h, q, nch),
+      copy_span<kNP, LP, 3 * kRY * 32>(&S.s.b.ft[slot][h][0][0][0], fac + fac_slab<kRY>(32, blockIdx.x, h, q, nch),
                                   3 * kRY * 32, p);
     }
   };
@@ -519,13 +537,8 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
           // factors are slab cell n-1-s (the forward pass ran the other way)
           const int n = r1 - r0, rb = h ? 0 : n - 1, rs = h ? 1 : -1;
           auto F = [&](int f, int s) { return S.s.b.ft[slot][h][f][n - 1 - s][lane]; };
-          auto xs = [&](int s) { return S.xs[lane][r0 + rb + rs * s - (m - 2)]; };
           auto put = [&](int s, LP x) { X[(rb + rs * s) * 32 + lane] = x; };
-          auto is_seam = [&](int s) {
-            const int j = r0 + rb + rs * s;
-            return twisted && (h ? j <= m + 1 : j >= m - 2);
-          };
-          bs_chunk<LP, kRY>(x1, x2, n, twisted && (h ? r0 <= m + 1 : r1 > m - 2), F, is_seam, xs, put);
+          bs_chunk<LP, kRY>(x1, x2, n, F, put);
         }
       }
     } else {
@@ -631,7 +644,7 @@ template <class LP> struct XSmem {
 
 // DEV (the ensemble graphs): the step's band constants *Ld come from device
 // memory.
-template <class Mode, bool DEV = false>
+template <class Mode, bool DEV, bool GEN>
 __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
     k_xsweep(ModelK M, LineK<typename Mode::LP> Lp, const typename Mode::LP* __restrict__ ul,
              typename Mode::LP* __restrict__ rw, typename Mode::LP* __restrict__ fac,
@@ -645,7 +658,7 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
   const int p = threadIdx.x - 64;
   const int nx = M.nx, ny = M.ny;
   const int j0 = blockIdx.x * 32;
-  const int m = split_point<kCX>(nx);
+  const int m = split_point(nx);
   const bool twisted = m < nx;
   const int nch0 = (m + kCX - 1) / kCX, nch1 = twisted ? (nx - m + kCX - 1) / kCX : 0;
   const int nch = max(nch0, nch1);
@@ -703,12 +716,12 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
                 q[5 * kCX * 32] = R[s];
               };
               const bool edge = !(ia >= 2 && ia + kG + 1 < nx);
-              if (!L.ml.pl32)  // general exponents or the linear model
-                band_rows<LP, kG, true, false>(L, A, ia, ib, nx, out);
+              if (GEN)  // other exponents and models
+                band_rows<LP, kG, 0, true, false>(L, A, ia, ib, nx, out);
               else if (!edge)
-                band_rows<LP, kG, false, true>(L, A, ia, ib, nx, out);
+                band_rows<LP, kG, 0, false, true>(L, A, ia, ib, nx, out);
               else
-                band_rows<LP, kG, true, true>(L, A, ia, ib, nx, out);
+                band_rows<LP, kG, 0, true, true>(L, A, ia, ib, nx, out);
             }
           }
         }
@@ -718,7 +731,7 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
       if (q < nchh(h) && j0 + lane < ny) {
         const int c0 = c0_of(h, q), c1 = c1_of(h, q);
         const LP* B = &S.s.f.band[q & 1][h][0][0][0];
-        lu_chunk<LP, kCX>(lu, B, lane, c1 - c0, fac + fac_slab<kCX>(blockIdx.x, h, q, nch) + lane, pivot_bad);
+        lu_chunk<LP, kCX>(lu, B, lane, c1 - c0, fac + fac_slab<kCX>(32, blockIdx.x, h, q, nch) + lane, pivot_bad);
       }
     }
     __syncthreads();
@@ -738,7 +751,7 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
     for (int h = 0; h < 2; ++h) {
       const int q = nchh(h) - 1 - bq;
       if (q < 0) continue;
-      copy_span<LP, 3 * kCX * 32>(&S.s.b.ft[slot][h][0][0][0], fac + fac_slab<kCX>(blockIdx.x, h, q, nch),
+      copy_span<kNP, LP, 3 * kCX * 32>(&S.s.b.ft[slot][h][0][0][0], fac + fac_slab<kCX>(32, blockIdx.x, h, q, nch),
                                   3 * kCX * 32, p);
     }
     __pipeline_commit();
@@ -771,13 +784,8 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
           // its factors are slab cell n-1-s
           const int n = c1 - c0, cb = h ? 0 : n - 1, cs = h ? 1 : -1;
           auto F = [&](int f, int s) { return S.s.b.ft[slot][h][f][n - 1 - s][lane]; };
-          auto xs = [&](int s) { return S.xs[lane][c0 + cb + cs * s - (m - 2)]; };
           auto put = [&](int s, LP x) { S.s.b.xb[t & 1][h][cb + cs * s][lane] = x; };
-          auto is_seam = [&](int s) {
-            const int i = c0 + cb + cs * s;
-            return twisted && (h ? i <= m + 1 : i >= m - 2);
-          };
-          bs_chunk<LP, kCX>(x1, x2, n, twisted && (h ? c0 <= m + 1 : c1 > m - 2), F, is_seam, xs, put);
+          bs_chunk<LP, kCX>(x1, x2, n, F, put);
         }
       }
     } else {

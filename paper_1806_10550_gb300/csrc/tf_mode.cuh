@@ -19,8 +19,66 @@ template <class Mode> struct Launch {
   static constexpr size_t smem_stencil = sizeof(StencilSmem<HP, 16, 16>);
   static constexpr size_t smem_rhs = sizeof(RhsSmem<HP, 32>);
   static constexpr bool kF32B = std::is_same<Mode, ModeF32B>::value;
-  static constexpr size_t smem_x = sizeof(XSmem<LP>);
-  static constexpr size_t smem_y = sizeof(YSmem<LP>);
+  // The kernel, threads and shared memory of a sweep (DIR 0: x, 1: y) in
+  // blocks of nl lines, and its launch.  DEV, GEN: see k_ysweep.
+  template <int NL, int DIR> static constexpr size_t smem_n = sizeof(NarrowSmem<LP, NL, DIR>);
+  static constexpr size_t smem_x = sizeof(XSmem<LP>), smem_y = sizeof(YSmem<LP>);
+  // whether any film runs in blocks of 32 lines (see sweep_lines and set_lines)
+  template <bool GEN> static constexpr bool kWide = !(kF32B && GEN);
+  template <int NL, bool DEV, bool GEN>
+  static void narrow_x(tf_ctx& c, const LineK<LP>& L, const LP* ul, const LineK<LP>* Ld, cudaStream_t s) {
+    k_narrow_sweep<Mode, NL, 0, DEV, GEN><<<c.grid_x, NarrowCfg<LP, NL>::NT, smem_n<NL, 0>, s>>>(
+        c.mk, L, nullptr, ul, (LP*)c.w, (LP*)c.fac_x, nullptr, nullptr, c.px + c.n_rhs_parts, nullptr, Ld, nullptr);
+  }
+  template <int NL, bool DEV, bool GEN>
+  static void narrow_y(tf_ctx& c, const LineK<LP>& L, const double* u, const LP* ul, double* un, double* v,
+                       const LineK<LP>* Ld, const double* const* uio, cudaStream_t s) {
+    k_narrow_sweep<Mode, NL, 1, DEV, GEN><<<c.grid_y, NarrowCfg<LP, NL>::NT, smem_n<NL, 1>, s>>>(
+        c.mk, L, u, ul, (LP*)c.w, (LP*)c.fac_y, un, v, nullptr, c.py, Ld, uio);
+  }
+  template <bool DEV, bool GEN>
+  static void launch_x(tf_ctx& c, const LineK<LP>& L, const LP* ul, const LineK<LP>* Ld, cudaStream_t s) {
+    switch (c.nlx) {
+      case 4: return narrow_x<4, DEV, GEN>(c, L, ul, Ld, s);
+      case 8: return narrow_x<8, DEV, GEN>(c, L, ul, Ld, s);
+      case 16: return narrow_x<16, DEV, GEN>(c, L, ul, Ld, s);
+      default:
+        if constexpr (kWide<GEN>)
+          k_xsweep<Mode, DEV, GEN><<<c.grid_x, kSweepThreads, smem_x, s>>>(c.mk, L, ul, (LP*)c.w, (LP*)c.fac_x,
+                                                                         c.px + c.n_rhs_parts, Ld);
+    }
+  }
+  template <bool DEV, bool GEN>
+  static void launch_y(tf_ctx& c, const LineK<LP>& L, const double* u, const LP* ul, double* un, double* v,
+                       const LineK<LP>* Ld, const double* const* uio, cudaStream_t s) {
+    switch (c.nly) {
+      case 4: return narrow_y<4, DEV, GEN>(c, L, u, ul, un, v, Ld, uio, s);
+      case 8: return narrow_y<8, DEV, GEN>(c, L, u, ul, un, v, Ld, uio, s);
+      case 16: return narrow_y<16, DEV, GEN>(c, L, u, ul, un, v, Ld, uio, s);
+      default:
+        if constexpr (kWide<GEN>)
+          k_ysweep<Mode, DEV, GEN><<<c.grid_y, kSweepThreads, smem_y, s>>>(c.mk, L, u, ul, (const LP*)c.w, (LP*)c.fac_y,
+                                                                         un, v, c.py, Ld, uio);
+    }
+  }
+  // Dynamic shared memory of a sweep kernel; two blocks share an SM only with
+  // the largest shared carveout.
+  template <class K> static cudaError_t allow(K k, size_t smem) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return e ? e : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  }
+  template <int NL, bool DEV, bool GEN> static cudaError_t prepare_narrow() {
+    cudaError_t e = allow(k_narrow_sweep<Mode, NL, 0, DEV, GEN>, smem_n<NL, 0>);
+    return e ? e : allow(k_narrow_sweep<Mode, NL, 1, DEV, GEN>, smem_n<NL, 1>);
+  }
+  template <bool DEV, bool GEN> static cudaError_t prepare_sweeps() {
+    cudaError_t e;
+    if constexpr (kWide<GEN>) {
+      if ((e = allow(k_xsweep<Mode, DEV, GEN>, smem_x)) || (e = allow(k_ysweep<Mode, DEV, GEN>, smem_y))) return e;
+    }
+    if ((e = prepare_narrow<4, DEV, GEN>()) || (e = prepare_narrow<8, DEV, GEN>())) return e;
+    return prepare_narrow<16, DEV, GEN>();
+  }
 
   static StepK step(const tf_ctx& c, double dt) {
     StepK k;
@@ -37,21 +95,12 @@ template <class Mode> struct Launch {
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsResidual>, A, (int)smem_rhs))) return e;
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsExplicit>, A, (int)smem_rhs))) return e;
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsBoth>, A, (int)smem_rhs))) return e;
-    if ((e = cudaFuncSetAttribute(k_xsweep<Mode>, A, (int)smem_x))) return e;
-    if ((e = cudaFuncSetAttribute(k_ysweep<Mode>, A, (int)smem_y))) return e;
-    // the sweeps run two blocks per SM only with the largest shared carveout
+    if ((e = prepare_sweeps<false, false>()) || (e = prepare_sweeps<false, true>())) return e;
     const cudaFuncAttribute C = cudaFuncAttributePreferredSharedMemoryCarveout;
-    if ((e = cudaFuncSetAttribute(k_xsweep<Mode>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
-    if ((e = cudaFuncSetAttribute(k_ysweep<Mode>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsExplicit>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsBoth>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
     if constexpr (kF32B) {
-      if ((e = part::prepare())) return e;
-      // the sweeps of the ensemble graphs (constants from device memory)
-      if ((e = cudaFuncSetAttribute(k_xsweep<Mode, true>, A, (int)smem_x))) return e;
-      if ((e = cudaFuncSetAttribute(k_ysweep<Mode, true>, A, (int)smem_y))) return e;
-      if ((e = cudaFuncSetAttribute(k_xsweep<Mode, true>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
-      if ((e = cudaFuncSetAttribute(k_ysweep<Mode, true>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
+      if ((e = part::prepare()) || (e = prepare_sweeps<true, false>())) return e;
     }
     return cudaFuncSetAttribute(k_rhs<Mode, kRhsResidual>, C, (int)cudaSharedmemCarveoutMaxShared);
   }
@@ -112,13 +161,16 @@ template <class Mode> struct Launch {
   static const LP* film_lp(const tf_ctx& c, const double* u_k) {
     return sizeof(LP) == sizeof(double) ? (const LP*)u_k : (const LP*)c.ulp;
   }
+  static bool power32(const tf_ctx& c) { return c.mk.model == 0 && c.mk.n == 3 && c.mk.m == 2; }
   static cudaError_t xsweep_c(tf_ctx& c, double dt, const double* u_k) {
     if constexpr (kF32B) {
       if (c.part) return part::xsweep(c, dt);
     }
-    k_xsweep<Mode><<<c.grid_x, kSweepThreads, smem_x, c.stream>>>(c.mk, line_consts<LP>(c.mk, step(c, dt)),
-                                                       film_lp(c, u_k), (LP*)c.w,
-                                                       (LP*)c.fac_x, c.px + c.n_rhs_parts);
+    const LineK<LP> L = line_consts<LP>(c.mk, step(c, dt));
+    if (power32(c))
+      launch_x<false, false>(c, L, film_lp(c, u_k), nullptr, c.stream);
+    else
+      launch_x<false, true>(c, L, film_lp(c, u_k), nullptr, c.stream);
     return cudaGetLastError();
   }
   static cudaError_t ysweep_c(tf_ctx& c, const double* u_k, double dt, double* u_next,
@@ -126,10 +178,11 @@ template <class Mode> struct Launch {
     if constexpr (kF32B) {
       if (c.part) return part::ysweep(c, u_k, dt, u_next, v_out);
     }
-    k_ysweep<Mode><<<c.grid_y, kSweepThreads, smem_y, c.stream>>>(c.mk, line_consts<LP>(c.mk, step(c, dt)),
-                                                       u_k, film_lp(c, u_k),
-                                                       (const LP*)c.w,
-                                                       (LP*)c.fac_y, u_next, v_out, c.py);
+    const LineK<LP> L = line_consts<LP>(c.mk, step(c, dt));
+    if (power32(c))
+      launch_y<false, false>(c, L, u_k, film_lp(c, u_k), u_next, v_out, nullptr, nullptr, c.stream);
+    else
+      launch_y<false, true>(c, L, u_k, film_lp(c, u_k), u_next, v_out, nullptr, nullptr, c.stream);
     return cudaGetLastError();
   }
   // The whole run of an ensemble film as one graph (FP32-bulk, (3, 2) power
@@ -162,11 +215,8 @@ template <class Mode> struct Launch {
       };
       // one Newton iteration's sweeps and reductions
       auto sweeps = [&]() {
-        k_xsweep<Mode, true><<<c.grid_x, kSweepThreads, smem_x, s>>>(c.mk, l0, (const LP*)c.ulp, (LP*)c.w,
-                                                                     (LP*)c.fac_x, c.px + c.n_rhs_parts, &e->line);
-        k_ysweep<Mode, true><<<c.grid_y, kSweepThreads, smem_y, s>>>(c.mk, l0, nullptr, (const LP*)c.ulp,
-                                                                     (const LP*)c.w, (LP*)c.fac_y, nullptr, nullptr,
-                                                                     c.py, &e->line, &e->p.uk);
+        launch_x<true, false>(c, l0, (const LP*)c.ulp, &e->line, s);
+        launch_y<true, false>(c, l0, nullptr, (const LP*)c.ulp, nullptr, nullptr, &e->line, &e->p.uk, s);
         k_ens_iter<<<1, 256, 0, s>>>(c.px, c.n_rhs_parts + c.grid_x, c.py, c.grid_y, c.dsc, e, hi);
       };
       if ((err = cudaGraphCreate(&g, 0))) return fail(err);

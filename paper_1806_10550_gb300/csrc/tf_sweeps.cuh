@@ -219,15 +219,11 @@ __device__ __forceinline__ bool seam(const LUState<LP>& S, const LUState<LP>& R,
   return solve4(A, b, x);
 }
 
-// Where each line splits: the first half covers cells [0, m) with m a
-// multiple of the chunk length C near n/2; twisting needs m >= 2 and
-// n - m >= 2.
-template <int C> __host__ __device__ __forceinline__ int split_point(int n) {
-  const int nch = (n + C - 1) / C;
-  const int m = ((nch + 1) / 2) * C;
-  if (m >= n - 1 || m < 2) return n;  // no second half
-  return m;
-}
+// Where each line splits: the first half covers cells [0, m), the second the
+// rest, each in chunks from its own end of the line.  In the middle, so that
+// neither half's chain is longer than it must be.  Lines shorter than 8 cells
+// are not split (twisting needs m >= 2 and n - m >= 2).
+__host__ __device__ __forceinline__ int split_point(int n) { return n < 8 ? n : (n + 1) / 2; }
 
 // Per-cell values for the band, read from an LP tile.  U(dr, dc) gives the
 // film at an offset from the cell; the tiles hold wall-reflected values, so
