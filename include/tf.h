@@ -375,9 +375,10 @@ int tf_adjoint_step(tf_ctx* ctx, const double* h_old, double dt, int K, const do
 
 /* Kernel time (ms, CUDA events) of the last tf_adjoint_step in this
  * process, by group: forward iterations, per-iterate tables and band
- * assembly, transposed line solves, x-line coefficient derivatives, y-line
- * coefficient derivatives, D derivatives, the copy of the kappa partial
- * sums.  n: entries wanted (up to 7).                                     */
+ * assembly, transposed line solves, the iterations' coefficient and D
+ * derivatives (x lines, y lines and D in one pass), 0 (the y lines' before
+ * they joined that pass), the explicit part's D derivative, the copy of the
+ * kappa partial sums.  n: entries wanted (up to 7).                        */
 int tf_adjoint_timing(double* ms, int n);
 
 /* ---- adjoint of a trajectory of fixed steps, with checkpoints ----------

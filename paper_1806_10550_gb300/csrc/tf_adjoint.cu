@@ -18,10 +18,12 @@
 // mobilities with two derivatives and the Laplacian, formed once per
 // iterate); see the comment above k_vjp_D.  Every face term depends on u
 // directly at its two cells and through the Laplacian at those cells, so
-// each transposed product is two gathers: one thread per cell over the
+// the transposed products are two gathers: one thread per cell over the
 // faces that touch it, then the transposed five-point Laplacian of the
 // collected Laplacian cotangents.  No atomics; every sum runs in a fixed
-// order.  FP64 throughout; the power-law and linear models.
+// order.  FP64 throughout; the power-law and linear models.  Everything here is
+// bound by FP64 instructions (0.55 us an instruction a cell at 512^2 over the
+// whole chip), so each kernel forms as few as its formulas allow.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdlib.h>
@@ -38,6 +40,7 @@ namespace {
 struct AdjK {
   int nx, ny, model, n, m;
   double ds, inv_ds, C, b, c0, c1, kappa, tdt;  // tdt = theta dt
+  double A1, B1;  // (n, m) = (3, 2): f1 = A1 - B1 / h
 };
 
 // Per-cell values of the iterate, formed once per iterate (FP64):
@@ -56,10 +59,18 @@ __global__ void k_tables(AdjK M, const double* __restrict__ u, Tables T) {
     T.f0[c] = M.c0;
     T.f1[c] = M.c1;
     T.d0[c] = T.d1[c] = T.e0[c] = T.e1[c] = 0.0;
+  } else if (M.n == 3 && M.m == 2) {
+    const double s = tf::rcp3(h), h2 = h * h, d1 = M.B1 * (s * s);
+    T.f0[c] = M.C * (h2 * h);
+    T.f1[c] = M.A1 - M.B1 * s;
+    T.d0[c] = 3.0 * M.C * h2;
+    T.d1[c] = d1;
+    T.e0[c] = 6.0 * M.C * h;
+    T.e1[c] = -2.0 * (d1 * s);
   } else {
     // Pi' = kappa (m r^m - n r^n)/h, Pi'' = kappa (n(n+1) r^n - m(m+1) r^m)/h^2,
     // Pi''' = kappa (m(m+1)(m+2) r^m - n(n+1)(n+2) r^n)/h^3, r = b/h
-    const double ih = 1.0 / h, r = M.b * ih;
+    const double ih = tf::rcp3(h), r = M.b * ih;
     double rm = 1.0, rn = 1.0;
     for (int q = 0; q < M.m; ++q) rm *= r;
     for (int q = 0; q < M.n; ++q) rn *= r;
@@ -83,46 +94,40 @@ __global__ void k_tables(AdjK M, const double* __restrict__ u, Tables T) {
   T.lap[c] = sl * M.inv_ds * M.inv_ds;
 }
 
-// d(along-line second difference at line cell c)/d(u at line cell col),
-// reflection at the ends of a line of n cells, times ds^2.
-__device__ __forceinline__ double dlap_line(int c, int col, int n) {
-  if (col == c + 1) return c < n - 1 ? 1.0 : 0.0;
-  if (col == c - 1) return c > 0 ? 1.0 : 0.0;
-  if (col == c) return -(double)((c < n - 1) + (c > 0));
-  return 0.0;
-}
-
 // Row of I + theta dt J along a line (DIR 0: x, the line is row j; DIR 1: y,
 // column i) at the line cell t = i or j: band[d] is the coefficient of line
-// cell t + d - 2.  Face between line cells p and q = p + 1: the flux
-// derivative has f0'/2 gL and f1'/2 gU on p and q (gL = (L_q - L_p)/ds with
-// the full Laplacian, gU = (u_q - u_p)/ds), fbar0 (dLline_q - dLline_p)/ds
-// over columns p-1..p+2, and -+fbar1/ds on p, q; row p gets +theta dt dF/ds,
-// row q -theta dt dF/ds.
+// cell t + d - 2.  The derivative of the flux through the face of line cells
+// p and q = p + 1, times theta dt / ds, over the columns p-1 .. q+1 is
+//   (-w_p c3, (2 + w_p) c3 + t_p - Bd, -(2 + w_q) c3 + t_q + Bd, w_q c3),
+// c3 = theta dt (f0_p + f0_q)/(2 ds^4), Bd = theta dt (f1_p + f1_q)/(2 ds^2),
+// t = theta dt (f0' dL + f1' du)/(2 ds^2) with the differences dL, du of the full
+// Laplacian and the height over the face, and w_p (w_q) 1 where p (q) has
+// another neighbour outward, else 0; row p gets it, row q its negative.
 template <int DIR>
-__device__ void row_band(const AdjK& M, const double* __restrict__ u, const Tables& T, int i, int j,
-                         double (&band)[5]) {
+__device__ __forceinline__ void row_band(const AdjK& M, const double* __restrict__ u, const Tables& T, int i, int j,
+                                         double (&band)[5]) {
   const int n = DIR == 0 ? M.nx : M.ny, t = DIR == 0 ? i : j;
   const size_t c = (size_t)j * M.nx + i, step = DIR == 0 ? 1 : (size_t)M.nx;
-  for (int d = 0; d < 5; ++d) band[d] = d == 2 ? 1.0 : 0.0;
-  for (int side = 0; side < 2; ++side) {
-    const int p = side == 0 ? t - 1 : t, q = p + 1;
-    if (p < 0 || q >= n) continue;
-    const size_t cp = side == 0 ? c - step : c, cq = cp + step;
-    const double fb0 = 0.5 * (T.f0[cp] + T.f0[cq]), fb1 = 0.5 * (T.f1[cp] + T.f1[cq]);
-    const double gL = M.inv_ds * (T.lap[cq] - T.lap[cp]), gU = M.inv_ds * (u[cq] - u[cp]);
-    const double sgn = side == 0 ? -1.0 : 1.0;  // row t is q (side 0) or p (side 1)
-    const double coef = sgn * M.tdt * M.inv_ds;
-    for (int a = 0; a < 4; ++a) {
-      const int col = p - 1 + a;
-      if (col < 0 || col >= n) continue;
-      const double dl = (dlap_line(q, col, n) - dlap_line(p, col, n)) * M.inv_ds * M.inv_ds * M.inv_ds;
-      double v = dl * fb0;
-      if (col == p) v += 0.5 * T.d0[cp] * gL + 0.5 * T.d1[cp] * gU - M.inv_ds * fb1;
-      if (col == q) v += 0.5 * T.d0[cq] * gL + 0.5 * T.d1[cq] * gU + M.inv_ds * fb1;
-      band[col - t + 2] += coef * v;
-    }
-  }
+  const double k1 = 0.5 * M.tdt * (M.inv_ds * M.inv_ds), k3 = k1 * (M.inv_ds * M.inv_ds);
+  const double f0 = T.f0[c], f1 = T.f1[c], d0 = k1 * T.d0[c], d1 = k1 * T.d1[c], lp = T.lap[c], uc = u[c];
+  double lo[4] = {0.0, 0.0, 0.0, 0.0}, hi[4] = {0.0, 0.0, 0.0, 0.0};
+  auto face = [&](size_t o, bool up, bool pl, bool qr, double (&F)[4]) {  // o the other cell; up: it is q
+    const double c3 = k3 * (f0 + T.f0[o]), Bd = k1 * (f1 + T.f1[o]);
+    const double dL = up ? T.lap[o] - lp : lp - T.lap[o], du = up ? u[o] - uc : uc - u[o];
+    const double tc = d0 * dL + d1 * du, to = k1 * (T.d0[o] * dL + T.d1[o] * du);
+    const double tp = up ? tc : to, tq = up ? to : tc;
+    F[0] = pl ? -c3 : 0.0;
+    F[1] = (pl ? 3.0 : 2.0) * c3 + (tp - Bd);
+    F[2] = (qr ? -3.0 : -2.0) * c3 + (tq + Bd);
+    F[3] = qr ? c3 : 0.0;
+  };
+  if (t > 0) face(c - step, false, t > 1, t + 1 < n, lo);
+  if (t + 1 < n) face(c + step, true, t > 0, t + 2 < n, hi);
+  band[0] = -lo[0];
+  band[1] = hi[0] - lo[1];
+  band[2] = 1.0 + (hi[1] - lo[2]);
+  band[3] = hi[2] - lo[3];
+  band[4] = hi[3];
 }
 
 // ---- transposed derivative products, hand-derived (two passes) ----------
@@ -150,7 +155,10 @@ __device__ void row_band(const AdjK& M, const double* __restrict__ u, const Tabl
 // Pass 1 (one thread per cell j, over the faces that touch j): the direct
 // u_j terms go to ubar_j, the L_j terms to Lbar_j, and the kappa terms of
 // the faces whose p is j to a per-block sum.  Pass 2: ubar_j += the
-// transposed five-point Laplacian of Lbar (symmetric, with reflection).
+// transposed five-point Laplacian of Lbar (symmetric, with reflection).  An
+// iteration's three products (the y lines, the x lines and D) share their
+// faces' values: one pass 1 forms them all and one pass 2 follows (512^2: 115
+// us an iteration against 193 for a pass pair each).
 
 struct FaceVals {
   double up, uq, f0p, f0q, f1p, f1q, d0p, d0q, d1p, d1q, e0p, e0q, e1p, e1q, gL, gU;
@@ -229,51 +237,59 @@ __global__ void __launch_bounds__(kVjpThreads) k_vjp_D(AdjK M, const double* __r
   block_sum_to(dk, part);
 }
 
-// A line row along DIR: ubar_j += scale ([d_u (A(u) w)]^T lambda)_j (direct
-// part), Lbar_j = its L_j part, part[block] = scale lambda^T d(A w)/dkappa.
-template <int DIR>
-__global__ void __launch_bounds__(kVjpThreads) k_vjp_line(AdjK M, const double* __restrict__ u, Tables T,
-                                                           const double* __restrict__ w,
-                                                           const double* __restrict__ lam, double scale,
-                                                           double* __restrict__ ubar, double* __restrict__ Lbar,
-                                                           double* __restrict__ part) {
+// The three products of an iteration: ubar_j becomes ubar_j - lx_j plus the
+// direct parts of -([d_u (A_y v)]^T ly + [d_u (A_x w)]^T lx + theta dt D'^T lx)_j,
+// Lbar_j their L_j parts, bbar_j += lx_j, part[block] the kappa sum.  With
+// everything of a face halved and scaled by -theta dt (lambda_p - lambda_q)/ds
+// (h_line, h_D; the same along x, where both cotangents are lx):
+//   line  d0_c W3 + gL e0_c w_c + gU e1_c w_c + (d1_c dw -+ s1)/ds,  L: +-s0/ds
+//   D     d0_c gL + d1_c gU -+ (f1_p + f1_q)/ds,                  L: +-(f0_p + f0_q)/ds
+// (upper signs: c is p), dw = w_q - w_p, s0 = f0'_p w_p + f0'_q w_q, s1 with f1'.
+__global__ void __launch_bounds__(kVjpThreads)
+    k_vjp_iter(AdjK M, const double* __restrict__ u, Tables T, const double* __restrict__ W,
+               const double* __restrict__ V, const double* __restrict__ lx, const double* __restrict__ ly,
+               double* __restrict__ ubar, double* __restrict__ Lbar, double* __restrict__ bbar,
+               double* __restrict__ part) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-  double du = 0.0, dL = 0.0, dk = 0.0;
+  double dk = 0.0;
   if (i < M.nx) {
     const size_t c = (size_t)j * M.nx + i;
-    const int n = DIR == 0 ? M.nx : M.ny, t = DIR == 0 ? i : j;
-    const size_t step = DIR == 0 ? 1 : (size_t)M.nx;
-    const double inv_kappa = M.model == TF_MODEL_LINEAR ? 0.0 : 1.0 / M.kappa;
-    const double ids3 = M.inv_ds * M.inv_ds * M.inv_ds;
-    for (int side = 0; side < 2; ++side) {
-      const int pt = side == 0 ? t - 1 : t, qt = pt + 1;  // line indices of p, q
-      if (pt < 0 || qt >= n) continue;
-      const size_t p = c - (size_t)(t - pt) * step, q = p + step;
-      const FaceVals v = face_vals(M, u, T, p, q);
-      const double wp = w[p], wq = w[q];
-      // W3: the along-line third difference of w over columns p-1..p+2
-      double W3 = 0.0;
-      for (int a = 0; a < 4; ++a) {
-        const int col = pt - 1 + a;
-        if (col < 0 || col >= n) continue;
-        const double dl = (dlap_line(qt, col, n) - dlap_line(pt, col, n)) * ids3;
-        W3 += dl * w[(size_t)((long long)c + (long long)(col - t) * (long long)step)];
-      }
-      const double fb1 = 0.5 * (v.f1p + v.f1q);
-      const double s0 = v.d0p * wp + v.d0q * wq, s1 = v.d1p * wp + v.d1q * wq;
-      const double mu = scale * M.tdt * (lam[p] - lam[q]) * M.inv_ds;
-      if (side == 0) {  // c is q
-        du += mu * (0.5 * v.d0q * W3 + 0.5 * v.gL * v.e0q * wq + 0.5 * v.gU * v.e1q * wq +
-                    0.5 * v.d1q * (wq - wp) * M.inv_ds + 0.5 * s1 * M.inv_ds);
-        dL += mu * 0.5 * s0 * M.inv_ds;
-      } else {  // c is p
-        du += mu * (0.5 * v.d0p * W3 + 0.5 * v.gL * v.e0p * wp + 0.5 * v.gU * v.e1p * wp +
-                    0.5 * v.d1p * (wq - wp) * M.inv_ds - 0.5 * s1 * M.inv_ds);
-        dL -= mu * 0.5 * s0 * M.inv_ds;
-        dk += mu * (0.5 * v.gU * s1 + fb1 * (wq - wp) * M.inv_ds) * inv_kappa;
+    const double ids = M.inv_ds, ids3 = ids * (ids * ids), hs = -0.5 * M.tdt * ids;
+    const double uc = u[c], f0c = T.f0[c], f1c = T.f1[c], d0c = T.d0[c], d1c = T.d1[c], lc = T.lap[c];
+    const double e0c = T.e0[c], e1c = T.e1[c], lxc = lx[c], lyc = ly[c];
+    double du = 0.0, dL = 0.0;
+#pragma unroll
+    for (int dir = 0; dir < 2; ++dir) {
+      const int n = dir == 0 ? M.nx : M.ny, t = dir == 0 ? i : j;
+      const size_t step = dir == 0 ? 1 : (size_t)M.nx;
+      const double* __restrict__ w = dir == 0 ? W : V;
+      const double wc = w[c], d0w = d0c * wc, d1w = d1c * wc, e0w = e0c * wc, e1w = e1c * wc;
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {  // 0: c is q, 1: c is p
+        if (side == 0 ? t == 0 : t + 1 >= n) continue;
+        const size_t o = side == 0 ? c - step : c + step;  // the other cell
+        const double wo = w[o];
+        const double dw = side == 0 ? wc - wo : wo - wc;
+        // third difference of w along the line, without the walls' neighbours
+        const double out = side == 0 ? (t > 1 ? wo - w[o - step] : 0.0) : (t + 2 < n ? w[o + step] - wo : 0.0);
+        const double in = side == 0 ? (t + 1 < n ? w[c + step] - wc : 0.0) : (t > 0 ? wc - w[c - step] : 0.0);
+        const double W3 = ids3 * ((out - dw) + (in - dw));
+        const double gL = ids * (side == 0 ? lc - T.lap[o] : T.lap[o] - lc);
+        const double gU = ids * (side == 0 ? uc - u[o] : u[o] - uc);
+        const double s0 = d0w + T.d0[o] * wo, s1 = d1w + T.d1[o] * wo;
+        const double f0s = f0c + T.f0[o], f1s = f1c + T.f1[o];
+        const double hD = hs * (side == 0 ? lx[o] - lxc : lxc - lx[o]);
+        const double hl = dir == 0 ? hD : hs * (side == 0 ? ly[o] - lyc : lyc - ly[o]);
+        const double sg = side == 0 ? 1.0 : -1.0;
+        du += hl * (d0c * W3 + (gL * e0w + (gU * e1w + ids * (d1c * dw + sg * s1))));
+        du += hD * (d0c * gL + (d1c * gU + (sg * ids) * f1s));
+        dL += (sg * ids) * (hl * s0 + hD * f0s);
+        if (side == 1) dk += hl * (gU * s1 + f1s * (ids * dw)) + hD * (f1s * gU);
       }
     }
-    ubar[c] += du;
+    dk *= M.model == TF_MODEL_LINEAR ? 0.0 : 1.0 / M.kappa;
+    ubar[c] = (ubar[c] - lxc) + du;
+    bbar[c] += lxc;
     Lbar[c] = dL;
   }
   block_sum_to(dk, part);
@@ -398,7 +414,7 @@ __global__ void __launch_bounds__(2 * kSolveLines) k_solve_t(int nx, int ny, con
           trow(k + 6, p_lo2[sl], p_lo1[sl], p_dg[sl], p_u1[sl], p_u2[sl]);
           p_y[sl] = r[idx(row_of(k + 6))];
         }
-        const double inv = 1.0 / a_dg;
+        const double inv = tf::rcp3(a_dg);
         if (k + 1 < nrows) {
           const double l = b_lo1 * inv;
           b_dg -= l * a_u1;
@@ -474,7 +490,7 @@ __global__ void __launch_bounds__(2 * kSolveLines) k_solve_t(int nx, int ny, con
 #pragma unroll 4
   for (int k = npiv - 1; k >= 0; --k) {
     const size_t ck = idx(row_of(k));
-    const double xv = (sy[ck] - s1[ck] * x1 - s2[ck] * x2) * sd[ck];
+    const double xv = ((sy[ck] - s2[ck] * x2) - s1[ck] * x1) * sd[ck];  // the newest value last
     x[ck] = xv;
     x2 = x1;
     x1 = xv;
@@ -553,7 +569,7 @@ struct RevWork {
 int rev_workspace(tf_ctx* c, int K, bool iterates, RevWork* w) {
   const size_t N = c->N;
   w->npart = ((c->p.nx + kVjpThreads - 1) / kVjpThreads) * c->p.ny;
-  w->nkl = 3 * K + 1;
+  w->nkl = K + 1;
   const size_t rev = 19 * N + (size_t)w->npart * w->nkl;
   const size_t bytes = (rev + (iterates ? (size_t)3 * K * N : 0)) * sizeof(double);
   if (c->adj_bytes < bytes) {
@@ -621,6 +637,8 @@ int adj_reverse(tf_ctx* c, const RevWork& R, const double* const* U, const doubl
   M.c0 = c->p.c0;
   M.c1 = c->p.c1;
   M.kappa = c->kappa;
+  M.A1 = c->mk.A1;
+  M.B1 = c->mk.B1;
   const double theta = c->p.theta;
   M.tdt = theta * dt;
 
@@ -646,10 +664,6 @@ int adj_reverse(tf_ctx* c, const RevWork& R, const double* const* U, const doubl
     t = T.begin(kGSolve);
     k_solve_t<1><<<nl_y, 2 * kSolveLines, 0, st>>>(nx, ny, band, g_h, lam_y, scratch);
     T.end(t);
-    t = T.begin(kGLineY);
-    k_vjp_line<1><<<gv, bv, 0, st>>>(M, uk, Tb, V[k], lam_y, -1.0, g_h, Lbar, part + (size_t)(kl++) * npart);
-    k_lap_t<<<g2, b2, 0, st>>>(M, Lbar, g_h);
-    T.end(t);
     // w_k = A_x(u_k)^-1 (-G(u_k))
     t = T.begin(kGBand);
     k_band<0><<<g2, b2, 0, st>>>(M, uk, Tb, band);
@@ -657,15 +671,9 @@ int adj_reverse(tf_ctx* c, const RevWork& R, const double* const* U, const doubl
     t = T.begin(kGSolve);
     k_solve_t<0><<<nl_x, 2 * kSolveLines, 0, st>>>(nx, ny, band, lam_y, lam_x, scratch);
     T.end(t);
+    // both lines' coefficients and -G(u_k) = -u_k - theta dt D(u_k) + b
     t = T.begin(kGLineX);
-    k_vjp_line<0><<<gv, bv, 0, st>>>(M, uk, Tb, W[k], lam_x, -1.0, g_h, Lbar, part + (size_t)(kl++) * npart);
-    k_lap_t<<<g2, b2, 0, st>>>(M, Lbar, g_h);
-    T.end(t);
-    // -G(u_k) = -u_k - theta dt D(u_k) + b
-    k_axpy<<<nb, 256, 0, st>>>(N, -1.0, lam_x, g_h);
-    k_axpy<<<nb, 256, 0, st>>>(N, 1.0, lam_x, bbar);
-    t = T.begin(kGD);
-    k_vjp_D<<<gv, bv, 0, st>>>(M, uk, Tb, lam_x, -M.tdt, g_h, Lbar, part + (size_t)(kl++) * npart);
+    k_vjp_iter<<<gv, bv, 0, st>>>(M, uk, Tb, W[k], V[k], lam_x, lam_y, g_h, Lbar, bbar, part + (size_t)(kl++) * npart);
     k_lap_t<<<g2, b2, 0, st>>>(M, Lbar, g_h);
     T.end(t);
   }
