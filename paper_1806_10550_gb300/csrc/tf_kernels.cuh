@@ -123,6 +123,28 @@ TF_HD float rcp(float x) {
   return 1.0f / x;
 #endif
 }
+// Reciprocal of the FP64 line solves and of the FP64 Jacobian's heights: a
+// float seed r0 of 1/x (relative error e = 1 - x r0 of about 2^-22, the
+// mantissas crossing between the formats with integer operations) and one
+// third-order step, 1/x = r0 (1 + e + e^2) + O(e^3): three FP64 operations,
+// rounded once at the end.  What bounds the FP64 sweeps is the number of FP64
+// instructions (a warp's takes 64 cycles of its sub-partition's pipe whatever
+// its lanes).  Zero, non-finite and extreme arguments take the division.
+__device__ __forceinline__ double rcp3(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ex = (hi >> 20) & 0x7ffu;
+  if (ex - 64u > 1918u) return 1.0 / x;  // the seed and 1/x are normal for exponents 64 .. 1982
+  const float m = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));  // |x| / 2^(ex - 1023), truncated
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(m));  // in [1/2, 1]
+  const unsigned rb = __float_as_uint(r);
+  const double r0 =
+      __hiloint2double((int)(((rb >> 3) + ((896u + 1023u - ex) << 20)) | (hi & 0x80000000u)), (int)(rb << 29));
+  const double e = fma(-x, r0, 1.0);
+  return fma(r0, fma(e, e, e), r0);
+}
+__device__ __forceinline__ float rcp3(float x) { return rcp(x); }
+
 TF_HD df64 rcp(df64 x) { return df_rcp(x); }
 
 template <class T> TF_HD T one();
@@ -146,16 +168,26 @@ template <class T> TF_HD T hpow_neg(const T& h, const T& s, int k) {
   return one<T>();
 }
 
+// The arithmetic that a mobility in T evaluates Pi in (see pi_model).
+template <class T> struct PiArith {
+  typedef double R;
+};
+template <> struct PiArith<float> {
+  typedef float R;
+};
+
 template <class T> struct MobC {
   T C, A1, B1, c0, c1, three, half;
   T dA1, dB1;  // (m-2) A1 and (n-2) B1
   int model, n, m;
   bool unitC;  // C == 1
   bool pl32;   // power law with (n, m) = (3, 2)
-  // NLC and polymer parameters (evaluated out of line, see pi_model)
-  double Cd, b, K, N, beta2, w, pC, pA1, pA12, pd;
+  // NLC and polymer parameters (see pi_model), in its arithmetic's type: a
+  // conversion in the kernel is an FP64-pipe instruction a cell
+  typename PiArith<T>::R Cd, b, K, N, beta2, iw, pC, pA1, pA12, pd;
 };
 template <class T> TF_HD MobC<T> mob_consts(const ModelK& M) {
+  typedef typename PiArith<T>::R R;
   MobC<T> c;
   c.C = from_f64<T>(M.C);
   c.A1 = from_f64<T>(M.A1);
@@ -171,16 +203,16 @@ template <class T> TF_HD MobC<T> mob_consts(const ModelK& M) {
   c.m = M.m;
   c.unitC = M.C == 1.0;
   c.pl32 = M.model == 0 && M.n == 3 && M.m == 2;
-  c.Cd = M.C;
-  c.b = M.b;
-  c.K = M.nlc_K;
-  c.N = M.nlc_N;
-  c.beta2 = M.nlc_beta * M.nlc_beta;
-  c.w = M.nlc_w;
-  c.pC = M.pol_C;
-  c.pA1 = M.pol_A1;
-  c.pA12 = M.pol_A1 - M.pol_A2;
-  c.pd = M.pol_d;
+  c.Cd = (R)M.C;
+  c.b = (R)M.b;
+  c.K = (R)M.nlc_K;
+  c.N = (R)M.nlc_N;
+  c.beta2 = (R)(M.nlc_beta * M.nlc_beta);
+  c.iw = (R)(1.0 / M.nlc_w);
+  c.pC = (R)M.pol_C;
+  c.pA1 = (R)M.pol_A1;
+  c.pA12 = (R)(M.pol_A1 - M.pol_A2);
+  c.pd = (R)M.pol_d;
   return c;
 }
 
@@ -250,23 +282,31 @@ template <class T> struct MobPair {
 //     Pi'' = 720 Cp/h^11 - 2A1/(pi h^5) + 2(A1 - A2)/(pi (h + d)^5).
 __host__ __device__ inline float r_tanh(float x) { return tanhf(x); }
 __host__ __device__ inline double r_tanh(double x) { return tanh(x); }
+__host__ __device__ inline float r_inv(float x) { return 1.0f / x; }
+__host__ __device__ inline double r_inv(double x) {
+#ifdef __CUDA_ARCH__
+  return rcp3(x);
+#else
+  return 1.0 / x;
+#endif
+}
 template <class R, class T>
 __host__ __device__ inline void pi_model(const MobC<T>& c, R h, R& d1, R& d2) {
-  const R ih = R(1) / h;
+  const R ih = r_inv(h);
   if (c.model == 3) {
     const R pi = R(3.14159265358979323846);
-    const R Cp = R(c.pC), A1 = R(c.pA1), A12 = R(c.pA12), ie = R(1) / (h + R(c.pd));
+    const R Cp = c.pC, A1 = c.pA1, A12 = c.pA12, ie = r_inv(h + c.pd);
     const R i2 = ih * ih, i4 = i2 * i2, i5 = i4 * ih, i10 = i5 * i5, e2 = ie * ie, e4 = e2 * e2;
     const R k = R(1) / (R(2) * pi);
     d1 = R(-72) * Cp * i10 + k * (A1 * i4 - A12 * e4);
     d2 = R(720) * Cp * i10 * ih - R(4) * k * (A1 * i5 - A12 * e4 * ie);
     return;
   }
-  const R b = R(c.b), K = R(c.K), N = R(c.N), be2 = R(c.beta2), iw = R(1) / R(c.w);
+  const R b = c.b, K = c.K, N = c.N, be2 = c.beta2, iw = c.iw;
   const R r = b * ih, r2 = r * r, r3 = r2 * r;
   const R t = r_tanh((h - R(2) * b) * iw), sech2 = R(1) - t * t;
   const R g = R(0.5) * (R(1) + t), dg = R(0.5) * sech2 * iw, d2g = -t * sech2 * iw * iw;
-  const R iD = R(1) / (h * h + be2), bmh = be2 - h * h;
+  const R iD = r_inv(h * h + be2), bmh = be2 - h * h;
   const R q = g * h * iD;
   const R dq = (dg * h + g * bmh * iD) * iD;
   const R d2q = (d2g * h + (R(2) * dg * bmh + g * R(2) * h * (h * h - R(3) * be2) * iD) * iD) * iD;
@@ -275,12 +315,6 @@ __host__ __device__ inline void pi_model(const MobC<T>& c, R h, R& d1, R& d2) {
 }
 // Height and values between T and the arithmetic R of pi_model: float stays
 // float; double and double-float evaluate in double.
-template <class T> struct PiArith {
-  typedef double R;
-};
-template <> struct PiArith<float> {
-  typedef float R;
-};
 __host__ __device__ inline double to_r(double x) { return x; }
 __host__ __device__ inline float to_r(float x) { return x; }
 __host__ __device__ inline double to_r(df64 x) { return f64_of_df(x); }
@@ -295,7 +329,7 @@ template <> __host__ __device__ inline df64 from_r<df64>(double x) { return df_o
 // evaluated out of line, so that kernels inline only the (n, m) = (3, 2)
 // power law.
 template <class T>
-__host__ __device__ __noinline__ MobPair<T> mobility_general(const MobC<T> c, const T h, const T s) {
+__host__ __device__ __noinline__ MobPair<T> mobility_general(const MobC<T>& c, const T h, const T s) {
   MobPair<T> r;
   if (c.model == 1) {
     r.a = c.c0;
@@ -307,7 +341,7 @@ __host__ __device__ __noinline__ MobPair<T> mobility_general(const MobC<T> c, co
     const R hr = to_r(h), h3 = hr * hr * hr;
     R d1, d2;
     pi_model<R>(c, hr, d1, d2);
-    r.a = from_r<T>(R(c.Cd) * h3);
+    r.a = from_r<T>(c.Cd * h3);
     r.b = from_r<T>(h3 * d1);
     return r;
   }
@@ -319,7 +353,7 @@ __host__ __device__ __noinline__ MobPair<T> mobility_general(const MobC<T> c, co
 }
 // f0' = 3 C h^2, f1' = -(m-2) A1 h^(1-m) + (n-2) B1 h^(1-n).
 template <class T>
-__host__ __device__ __noinline__ MobPair<T> mobility_d_general(const MobC<T> c, const T h, const T s) {
+__host__ __device__ __noinline__ MobPair<T> mobility_d_general(const MobC<T>& c, const T h, const T s) {
   MobPair<T> r;
   if (c.model == 1) {
     r.a = zero<T>();
@@ -331,7 +365,7 @@ __host__ __device__ __noinline__ MobPair<T> mobility_d_general(const MobC<T> c, 
     const R hr = to_r(h), h2 = hr * hr;
     R d1, d2;
     pi_model<R>(c, hr, d1, d2);
-    r.a = from_r<T>(R(3) * R(c.Cd) * h2);
+    r.a = from_r<T>(R(3) * c.Cd * h2);
     r.b = from_r<T>(R(3) * h2 * d1 + h2 * hr * d2);
     return r;
   }
@@ -346,15 +380,15 @@ template <class T> struct MobQuad {
   T f0, f1, d0, d1;
 };
 template <class T>
-__host__ __device__ __noinline__ MobQuad<T> mobility_model_all(const MobC<T> c, const T h) {
+__host__ __device__ __noinline__ MobQuad<T> mobility_model_all(const MobC<T>& c, const T h) {
   typedef typename PiArith<T>::R R;
   const R hr = to_r(h), h2 = hr * hr, h3 = h2 * hr;
   R d1, d2;
   pi_model<R>(c, hr, d1, d2);
   MobQuad<T> q;
-  q.f0 = from_r<T>(R(c.Cd) * h3);
+  q.f0 = from_r<T>(c.Cd * h3);
   q.f1 = from_r<T>(h3 * d1);
-  q.d0 = from_r<T>(R(3) * R(c.Cd) * h2);
+  q.d0 = from_r<T>(R(3) * c.Cd * h2);
   q.d1 = from_r<T>(R(3) * h2 * d1 + h3 * d2);
   return q;
 }
@@ -558,28 +592,6 @@ __device__ __forceinline__ void face_dF(const CellLP<LP>& P, const CellLP<LP>& Q
   dF[2] = -(LP(2) + wq) * c3 + h * sc * (Q.d0 * gL + Q.d1 * gU) + Bd;
   dF[3] = wq * c3;
 }
-
-// Reciprocal of the FP64 line solves and of the FP64 Jacobian's heights: a
-// float seed r0 of 1/x (relative error e = 1 - x r0 of about 2^-22, the
-// mantissas crossing between the formats with integer operations) and one
-// third-order step, 1/x = r0 (1 + e + e^2) + O(e^3): three FP64 operations,
-// rounded once at the end.  What bounds the FP64 sweeps is the number of FP64
-// instructions (a warp's takes 64 cycles of its sub-partition's pipe whatever
-// its lanes).  Zero, non-finite and extreme arguments take the division.
-__device__ __forceinline__ double rcp3(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned ex = (hi >> 20) & 0x7ffu;
-  if (ex - 64u > 1918u) return 1.0 / x;  // the seed and 1/x are normal for exponents 64 .. 1982
-  const float m = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));  // |x| / 2^(ex - 1023), truncated
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(m));  // in [1/2, 1]
-  const unsigned rb = __float_as_uint(r);
-  const double r0 =
-      __hiloint2double((int)(((rb >> 3) + ((896u + 1023u - ex) << 20)) | (hi & 0x80000000u)), (int)(rb << 29));
-  const double e = fma(-x, r0, 1.0);
-  return fma(r0, fma(e, e, e), r0);
-}
-__device__ __forceinline__ float rcp3(float x) { return rcp(x); }
 
 template <class LP> struct LUState {
   LP g1, d1, z1, g2, d2, z2;  // (gamma, delta, z) of rows i-1 and i-2
