@@ -567,10 +567,15 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
   c->grid_ry = (p->ny + 31) / 32;
   {
     // residual strips: segments of 64 rows, halved (down to 16) until the
-    // grid holds two waves of warps (about 24 resident per SM)
+    // grid holds two waves of warps (about 24 resident per SM), and further
+    // (down to 2) while it still fits in one (20 per SM): a row step takes a
+    // warp about a microsecond, so a small film's residual is as long as its
+    // segments (64^2: 17 us in segments of 16 rows)
     const long strips = (p->nx + tf::kRhsStripCols - 1) / tf::kRhsStripCols;
     int rows = 64;
-    while (rows > 16 && strips * ((p->ny + rows - 1) / rows) < 2L * 152 * 24) rows /= 2;
+    auto warps_at = [&](int r) { return strips * ((p->ny + r - 1) / r); };
+    while (rows > 16 && warps_at(rows) < 2L * kSMs * 24) rows /= 2;
+    while (rows > 2 && rows <= 16 && warps_at(rows / 2) <= (long)kSMs * 20) rows /= 2;
     const long warps = strips * ((p->ny + rows - 1) / rows);
     c->strip_n = (int)strips;
     c->strip_rows = rows;
@@ -587,6 +592,7 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
     c->n_px = a > b ? a : b;
   }
   c->n_py = c->grid_y > c->grid_stats ? c->grid_y : c->grid_stats;
+  if (c->packed_rhs && c->grid_pkx > c->n_py) c->n_py = c->grid_pkx;
   const size_t hp = c->ops->hp_bytes, lp = c->ops->lp_bytes;
   // factor scratch: one slab per sweep block, line half and chunk
   // (sized for blocks of 32, the most that a partly filled last block takes)
@@ -645,10 +651,9 @@ int tf_residual(tf_ctx* c, const double* h_k, const double* h_old, double dt, do
                 tf_norms* out) {
   if (!c || !h_k || !h_old || !isfinite(dt)) return TF_ERR_ARG;
   TF_CK(c->ops->explicit_part(*c, h_old, dt));
-  TF_CK(c->ops->residual_g(*c, h_k, dt, G ? G : c->ubuf));
-  tf::k_grid_stats<<<c->grid_stats, 256, 0, c->stream>>>(h_k, c->N, c->py);
-  TF_CK(cudaGetLastError());
-  int r = finalize(*c, c->grid_st_x * c->grid_st_y, c->grid_stats);
+  int npx = 0, npy = 0;
+  TF_CK(c->ops->residual_g(*c, h_k, dt, G ? G : c->ubuf, &npx, &npy));
+  int r = finalize(*c, npx, npy);
   if (r) return r;
   if (out) {
     out->gnorm = c->hsc->gnorm;

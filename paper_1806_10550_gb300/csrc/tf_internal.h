@@ -28,7 +28,8 @@ struct Ops {
   cudaError_t (*explicit_part)(tf_ctx& c, const double* u_old, double dt);
   // explicit part plus the first iteration's right side (u_0 = u_old)
   cudaError_t (*explicit_rhs0)(tf_ctx& c, const double* u_old, double dt);
-  cudaError_t (*residual_g)(tf_ctx& c, const double* u_k, double dt, double* G);
+  // G to tf_residual's callers; the numbers of partial results in px and py
+  cudaError_t (*residual_g)(tf_ctx& c, const double* u_k, double dt, double* G, int* npx, int* npy);
   cudaError_t (*rhs)(tf_ctx& c, const double* u_k, double dt);
   cudaError_t (*xsweep)(tf_ctx& c, double dt, const double* u_k);
   cudaError_t (*ysweep)(tf_ctx& c, const double* u_k, double dt, double* u_next, double* v_out);

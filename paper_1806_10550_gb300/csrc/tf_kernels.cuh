@@ -244,8 +244,9 @@ template <class T> TF_HD LineK<T> line_consts(const ModelK& M, const StepK& K) {
 }
 // What a residual-stencil kernel forms: the residual of an iteration, the
 // explicit part of a step, or both from one D(u^n) (a step's first
-// iteration starts from u_0 = u^n).
-enum { kRhsResidual = 0, kRhsExplicit = 1, kRhsBoth = 2 };
+// iteration starts from u_0 = u^n), or the residual as tf_residual reports it
+// (G in FP64 with its norm, and the iterate's mass and least height).
+enum { kRhsResidual = 0, kRhsExplicit = 1, kRhsBoth = 2, kRhsReport = 3 };
 
 template <class T> struct RhsK {
   MobC<T> mc;
@@ -521,7 +522,7 @@ __device__ __forceinline__ HP stencil_dprime(const StencilSmem<HP, TR, TC>& S, i
 
 template <class Mode, int OUT_G>
 __global__ void __launch_bounds__(256)
-    k_stencil(ModelK M, StepK K, const double* __restrict__ u, typename Mode::HP* __restrict__ bn,
+    k_stencil(ModelK M, RhsK<typename Mode::HP> RK, const double* __restrict__ u, typename Mode::HP* __restrict__ bn,
               double* __restrict__ G, PartX* __restrict__ part) {
   typedef typename Mode::HP HP;
   constexpr int T = 16;
@@ -529,11 +530,9 @@ __global__ void __launch_bounds__(256)
   StencilSmem<HP, T, T>& S = *reinterpret_cast<StencilSmem<HP, T, T>*>(smem_raw);
   const int tid = threadIdx.y * T + threadIdx.x, nt = T * T;
   const int x0 = blockIdx.x * T, j0 = blockIdx.y * T;
-  const MobC<HP> mc = mob_consts<HP>(M);
-  const HP inv_ds2 = from_f64<HP>(M.inv_ds2);
   stencil_load(S, u, M, j0, x0, tid, nt);
   __syncthreads();
-  stencil_cells(S, mc, inv_ds2, tid, nt);
+  stencil_cells(S, RK.mc, RK.inv_ds2, tid, nt);
   __syncthreads();
   stencil_faces(S, M, j0, x0, tid, nt);
   __syncthreads();
@@ -545,13 +544,11 @@ __global__ void __launch_bounds__(256)
     HP dp = stencil_dprime(S, r, c);
     HP uc = S.u[r + 2][c + 2];
     if (OUT_G) {
-      HP scale = from_f64<HP>(0.5 * M.inv_ds2 * K.theta_dt);
-      HP Gv = (uc - bn[idx]) + scale * dp;
+      HP Gv = (uc - bn[idx]) + RK.gscale * dp;
       G[idx] = to_f64(Gv);
       g = fabs(to_f64(Gv));
     } else {
-      HP scale = from_f64<HP>(0.5 * M.inv_ds2 * K.expl_dt);
-      bn[idx] = uc - scale * dp;
+      bn[idx] = uc - RK.gscale * dp;
     }
   }
   if (OUT_G) {

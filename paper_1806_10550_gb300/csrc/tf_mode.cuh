@@ -119,9 +119,23 @@ template <class Mode> struct Launch {
                                                          (HP*)c.bn, nullptr, nullptr, nullptr);
     return cudaGetLastError();
   }
-  static cudaError_t residual_c(tf_ctx& c, const double* u_k, double dt, double* G) {
+  // G of tf_residual, the partial results of its norm and the film's mass and
+  // least height: *npx of them in c.px, *npy in c.py
+  static cudaError_t residual_c(tf_ctx& c, const double* u_k, double dt, double* G, int* npx, int* npy) {
+    if constexpr (kF32B) {
+      if (c.packed_rhs) {
+        *npx = *npy = c.grid_pkx;
+        k_rhs_strip<kRhsReport><<<c.grid_pkx, kST, 0, c.stream>>>(
+            c.mk, strip_consts(c.mk, step(c, dt), false), u_k, (HP*)c.bn, nullptr, nullptr, c.px, c.strip_n, c.strip_rows,
+            nullptr, nullptr, G, c.py);
+        return cudaGetLastError();
+      }
+    }
+    *npx = c.grid_st_x * c.grid_st_y;
+    *npy = c.grid_stats;
+    k_grid_stats<<<c.grid_stats, 256, 0, c.stream>>>(u_k, c.N, c.py);
     dim3 grid(c.grid_st_x, c.grid_st_y), block(16, 16);
-    k_stencil<Mode, 1><<<grid, block, smem_stencil, c.stream>>>(c.mk, step(c, dt), u_k, (HP*)c.bn,
+    k_stencil<Mode, 1><<<grid, block, smem_stencil, c.stream>>>(c.mk, rhs_consts<HP>(c.mk, step(c, dt)), u_k, (HP*)c.bn,
                                                                 G, c.px);
     return cudaGetLastError();
   }

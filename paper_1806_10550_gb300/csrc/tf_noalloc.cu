@@ -79,8 +79,8 @@ cudaError_t run(const tf::ModelK& mk, double theta, cudaStream_t s, const double
   dim3 grid((mk.nx + 15) / 16, (mk.ny + 15) / 16), block(16, 16);
   HP* bn = (HP*)scratch;
   tf::PartX* px = (tf::PartX*)(scratch + kPartOff);
-  tf::k_stencil<Mode, 0><<<grid, block, smem, s>>>(mk, K, h_old, bn, nullptr, nullptr);
-  tf::k_stencil<Mode, 1><<<grid, block, smem, s>>>(mk, K, h_k, bn, G, px);
+  tf::k_stencil<Mode, 0><<<grid, block, smem, s>>>(mk, tf::rhs_consts<HP>(mk, K, true), h_old, bn, nullptr, nullptr);
+  tf::k_stencil<Mode, 1><<<grid, block, smem, s>>>(mk, tf::rhs_consts<HP>(mk, K), h_k, bn, G, px);
   return cudaGetLastError();
 }
 

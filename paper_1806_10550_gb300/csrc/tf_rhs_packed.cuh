@@ -119,14 +119,21 @@ template <bool FAST> __device__ __forceinline__ df2 hdiff(df2 a, df2 b) {
   if constexpr (FAST) return d2(p_sub(a.hi, b.hi), p_sub(a.lo, b.lo));
   return d2_sub_u(a, b);
 }
-// 1/a for a positive double-float a (the refined MUFU reciprocal)
-__device__ __forceinline__ df2 d2_rcp_fast(df2 a) {
+// 1/a for a positive double-float a: the MUFU reciprocal refined by one step,
+// of second order, or of third (ACC)
+template <bool ACC> __device__ __forceinline__ df2 d2_rcp_fast(df2 a) {
   const float2 y = make_float2(rcp(a.hi.x), rcp(a.hi.y));
   // t = -(1 - a y) exactly: fma(a.hi, y, -1), then fma(a.lo, y, .)
   float2 t = p_fma(a.hi, y, p_splat(-1.0f));
   t = p_fma(a.lo, y, t);
+  if constexpr (ACC) t = p_fma(t, p_negz(t), t);  // t - t^2
   return d2(y, p_negz(p_mul(y, t)));
 }
+// products and sums of the residual: lazy, or normalised (ACC: the residual
+// that is reported, which callers difference further)
+template <bool ACC> __device__ __forceinline__ df2 m_mul(df2 a, df2 b) { return ACC ? d2_mul(a, b) : d2_mul_u(a, b); }
+template <bool ACC> __device__ __forceinline__ df2 m_add(df2 a, df2 b) { return ACC ? d2_add(a, b) : d2_add_u(a, b); }
+template <bool ACC> __device__ __forceinline__ df2 m_sub(df2 a, df2 b) { return ACC ? d2_norm(d2_sub_u(a, b)) : d2_sub_u(a, b); }
 
 // ---------------------------------------------------------------------------
 // the kernel
@@ -202,7 +209,7 @@ __device__ __forceinline__ bool strip_fast(unsigned lo, unsigned hi) {
 
 // Laplacian (unscaled), f0 and f1 ds^2 of the pair U with the rows above
 // (Um) and below (Up); (lh, ll) is the left neighbour's height, (rh, rl) the right one's
-template <bool FAST>
+template <bool FAST, bool ACC>
 __device__ __forceinline__ void strip_cells(const StripK& K, const df2& U, const df2& Um, const df2& Up, float lh,
                                             float ll, float rh, float rl, df2& lap, df2& f0, df2& f1) {
   const df2 E = d2(make_float2(U.hi.y, rh), make_float2(U.lo.y, rl));
@@ -216,9 +223,9 @@ __device__ __forceinline__ void strip_cells(const StripK& K, const df2& U, const
     l = d2_add_u(d2_add_u(d2_sub_u(E, U), d2_sub_u(Wn, U)), d2_add_u(d2_sub_u(Up, U), d2_sub_u(Um, U)));
   }
   lap = l;
-  const df2 h2 = d2_mul_u(U, U);
-  f0 = K.unitC ? d2_mul_u(h2, U) : d2_mul_u(d2_mul_u(d2_splat(K.C), h2), U);
-  f1 = d2_sub_u(d2_splat(K.A1s), d2_mul_u(d2_splat(K.B1s), d2_rcp_fast(U)));
+  const df2 h2 = m_mul<ACC>(U, U);
+  f0 = K.unitC ? m_mul<ACC>(h2, U) : m_mul<ACC>(m_mul<ACC>(d2_splat(K.C), h2), U);
+  f1 = m_sub<ACC>(d2_splat(K.A1s), m_mul<ACC>(d2_splat(K.B1s), d2_rcp_fast<ACC>(U)));
 }
 
 struct StripState {
@@ -231,12 +238,15 @@ struct StripState {
 // One row step: from the state at row j and the heights U2 of row j + 2,
 // G of row j (when `out`), then the state at row j + 1.  Returns max|G|
 // of the lane's cells.
+// (kRhsReport: G goes to Gout, and gmax takes the bits of max|G|.)
 template <int KIND, bool FAST>
 __device__ __forceinline__ float strip_step(StripState& s, const df2& U2, const df2& B, bool out, int j, int a,
                                             bool lane_out, const StripK& RK, int nx, int ny,
                                             df64* __restrict__ bn, float* __restrict__ rhs,
-                                            float* __restrict__ ulp) {
+                                            float* __restrict__ ulp, double* __restrict__ Gout,
+                                            unsigned long long& gmax) {
   constexpr unsigned F = 0xffffffffu;
+  constexpr bool ACC = KIND == kRhsReport;
   // x faces left of the lane's two cells, (a - 1 | a) and (a | a + 1), and
   // the x part of their divergence
   df2 dx = d2(p_splat(0.0f), p_splat(0.0f));
@@ -248,25 +258,25 @@ __device__ __forceinline__ float strip_step(StripState& s, const df2& U2, const 
     const df2 f1P = d2(make_float2(f1h, s.f1.hi.x), make_float2(f1l, s.f1.lo.x));
     const df2 lP = d2(make_float2(lph, s.lap.hi.x), make_float2(lpl, s.lap.lo.x));
     const df2 uP = d2(make_float2(s.Lh, s.U0.hi.x), make_float2(s.Ll, s.U0.lo.x));
-    df2 Fx = d2_add_u(d2_mul_u(d2_add_u(f0P, s.f0), d2_sub_u(s.lap, lP)),
-                      d2_mul_u(d2_add_u(f1P, s.f1), hdiff<FAST>(s.U0, uP)));
+    df2 Fx = m_add<ACC>(m_mul<ACC>(m_add<ACC>(f0P, s.f0), m_sub<ACC>(s.lap, lP)),
+                        m_mul<ACC>(m_add<ACC>(f1P, s.f1), hdiff<FAST>(s.U0, uP)));
     if (!(a - 1 >= 0 && a < nx)) Fx.hi.x = Fx.lo.x = 0.0f;
     if (!(a >= 0 && a + 1 < nx)) Fx.hi.y = Fx.lo.y = 0.0f;
     const float nh = __shfl_down_sync(F, Fx.hi.x, 1), nl = __shfl_down_sync(F, Fx.lo.x, 1);
-    dx = d2_sub_u(d2(make_float2(Fx.hi.y, nh), make_float2(Fx.lo.y, nl)), Fx);
+    dx = m_sub<ACC>(d2(make_float2(Fx.hi.y, nh), make_float2(Fx.lo.y, nl)), Fx);
   }
   // cell values of row j + 1
   const float l1h = __shfl_up_sync(F, s.U1.hi.y, 1), l1l = __shfl_up_sync(F, s.U1.lo.y, 1);
   const float r1h = __shfl_down_sync(F, s.U1.hi.x, 1), r1l = __shfl_down_sync(F, s.U1.lo.x, 1);
   df2 lap1, f01, f11;
-  strip_cells<FAST>(RK, s.U1, s.U0, U2, l1h, l1l, r1h, r1l, lap1, f01, f11);
+  strip_cells<FAST, ACC>(RK, s.U1, s.U0, U2, l1h, l1l, r1h, r1l, lap1, f01, f11);
   // the face between rows j and j + 1 (zero on the walls)
-  df2 FyP = d2_add_u(d2_mul_u(d2_add_u(s.f0, f01), d2_sub_u(lap1, s.lap)),
-                     d2_mul_u(d2_add_u(s.f1, f11), hdiff<FAST>(s.U1, s.U0)));
+  df2 FyP = m_add<ACC>(m_mul<ACC>(m_add<ACC>(s.f0, f01), m_sub<ACC>(lap1, s.lap)),
+                       m_mul<ACC>(m_add<ACC>(s.f1, f11), hdiff<FAST>(s.U1, s.U0)));
   if (!(j >= 0 && j + 1 < ny)) FyP = d2(p_splat(0.0f), p_splat(0.0f));
   float g = 0.0f;
   if (out && lane_out && a < nx) {
-    const df2 dp = d2_add_u(dx, d2_sub_u(FyP, s.FyM));
+    const df2 dp = m_add<ACC>(dx, m_sub<ACC>(FyP, s.FyM));
     const df2 uc = s.U0;
     const bool two = a + 1 < nx;
     const size_t idx = (size_t)j * nx + a;
@@ -287,23 +297,34 @@ __device__ __forceinline__ float strip_step(StripState& s, const df2& U2, const 
       }
       const df2 gs = KIND == kRhsBoth ? d2_splat(RK.gs2) : gscale;
       // -G = (b^n - u) - gs dp: the negation of G's operations, exactly
-      const df2 Gn = d2_norm(d2_sub_u(d2_sub_u(bv, uc), d2_mul_u(gs, dp)));
-      const float2 gl = p_add(Gn.hi, Gn.lo);
-      // FP32 film for the sweeps: the leading float of the double-float height
-      if (two && ((nx | a) & 1) == 0) {
-        *reinterpret_cast<float2*>(rhs + idx) = gl;
-        *reinterpret_cast<float2*>(ulp + idx) = uc.hi;
+      const df2 Gn = d2_norm(d2_sub_u(m_sub<ACC>(bv, uc), m_mul<ACC>(gs, dp)));
+      if constexpr (KIND == kRhsReport) {
+        auto put = [&](size_t k, float hi, float lo) {
+          const double G = f64_of_df(df_make(-hi, -lo));
+          Gout[k] = G;
+          const unsigned long long b = (unsigned long long)__double_as_longlong(G) & 0x7fffffffffffffffull;
+          if (b > gmax && b <= 0x7ff0000000000000ull) gmax = b;  // NaN is left out
+        };
+        put(idx, Gn.hi.x, Gn.lo.x);
+        if (two) put(idx + 1, Gn.hi.y, Gn.lo.y);
       } else {
-        rhs[idx] = gl.x;
-        ulp[idx] = uc.hi.x;
-        if (two) {
-          rhs[idx + 1] = gl.y;
-          ulp[idx + 1] = uc.hi.y;
+        const float2 gl = p_add(Gn.hi, Gn.lo);
+        // FP32 film for the sweeps: the leading float of the double-float height
+        if (two && ((nx | a) & 1) == 0) {
+          *reinterpret_cast<float2*>(rhs + idx) = gl;
+          *reinterpret_cast<float2*>(ulp + idx) = uc.hi;
+        } else {
+          rhs[idx] = gl.x;
+          ulp[idx] = uc.hi.x;
+          if (two) {
+            rhs[idx + 1] = gl.y;
+            ulp[idx + 1] = uc.hi.y;
+          }
         }
+        g = fabsf(gl.x);
+        const float ag = two ? fabsf(gl.y) : 0.0f;
+        if (!(ag <= g)) g = ag;
       }
-      g = fabsf(gl.x);
-      const float ag = two ? fabsf(gl.y) : 0.0f;
-      if (!(ag <= g)) g = ag;
     }
   }
   s.U0 = s.U1;
@@ -352,6 +373,9 @@ __device__ __forceinline__ void strip_copy_bn(float4* dst, const df64* __restric
 // KIND: kRhsResidual (G from u_k and the stored b^n), kRhsExplicit (b^n from
 // u^n) or kRhsBoth (b^n from u^n, stored, and G of the first iteration,
 // u_0 = u^n, from the same stored b^n -- what kRhsResidual would compute).
+// kRhsReport: G of kRhsResidual in FP64 to Gout, its norm in double, and mass
+// and least height of u_k to party (the heights pass through anyway): at 2048^2
+// it takes the place of a 16 x 16-tile kernel of 242 us and a pass of 14 us.
 // Warp w of the grid takes strip w % nstrip and rows [seg_rows * (w /
 // nstrip), + seg_rows); one partial result (max|G|) per block.
 // DEV (the ensemble graphs): the step's constants *RKd and the grid *ud come
@@ -360,7 +384,9 @@ template <int KIND, bool DEV = false>
 __global__ void __launch_bounds__(kST, 5)
     k_rhs_strip(ModelK M, StripK RKp, const double* __restrict__ up, df64* __restrict__ bn,
                 float* __restrict__ rhs, float* __restrict__ ulp, PartX* __restrict__ part, int nstrip,
-                int seg_rows, const StripK* __restrict__ RKd = nullptr, const double* const* __restrict__ ud = nullptr) {
+                int seg_rows, const StripK* __restrict__ RKd = nullptr, const double* const* __restrict__ ud = nullptr,
+                double* __restrict__ Gout = nullptr, PartY* __restrict__ party = nullptr) {
+  constexpr bool kB = KIND == kRhsResidual || KIND == kRhsReport;  // reads b^n
   const StripK& RK = DEV ? *RKd : RKp;
   const double* __restrict__ u = DEV ? *ud : up;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -369,6 +395,9 @@ __global__ void __launch_bounds__(kST, 5)
   const int nseg = (ny + seg_rows - 1) / seg_rows;
   __shared__ StripRing ring[kSWarps];
   float g = 0.0f;
+  unsigned long long gmax = 0ull, hmin = 0x7ff0000000000000ull;  // bits of max|G| and of the least height
+  Mass128 mass = {0ull, 0ull};
+  int nf = 0;
   if (w < nstrip * nseg) {
     const int x0 = (w % nstrip) * kSW, ja = (w / nstrip) * seg_rows;
     const int jb = min(ja + seg_rows, ny);
@@ -377,15 +406,27 @@ __global__ void __launch_bounds__(kST, 5)
     const bool inner = x0 - 2 >= 0 && x0 + kSW + 2 <= nx && (nx & 1) == 0 &&
                        (reinterpret_cast<uintptr_t>(u) & 15) == 0;
     StripRing& R = ring[warp];
+    auto stats = [&](double2 v) {  // the lane's pair of an output row
+      auto take = [&](double x) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+        if (!positive_finite_bits(x)) nf = 1;
+        else if (b < hmin) hmin = b;
+        mass_add(mass, (unsigned long long)fixed36_of_f64(x));
+      };
+      if (lane_out && a < nx) take(v.x);
+      if (lane_out && a + 1 < nx) take(v.y);
+    };
     // rows ja - 2 .. ja directly; rows ja + 1, ja + 2 (and b^n of rows ja,
     // ja + 1) queued
     unsigned lo0, hi0, lo1, hi1, lo2, hi2, lo3, hi3;
     const df2 Um2 = strip_conv(strip_load(u, nx, ny, ja - 2, a, inner), lo0, hi0);
     const df2 Um1 = strip_conv(strip_load(u, nx, ny, ja - 1, a, inner), lo1, hi1);
-    const df2 Ua = strip_conv(strip_load(u, nx, ny, ja, a, inner), lo2, hi2);
+    const double2 va = strip_load(u, nx, ny, ja, a, inner);
+    const df2 Ua = strip_conv(va, lo2, hi2);
+    if constexpr (KIND == kRhsReport) stats(va);
     for (int q = 1; q <= 2; ++q) {
       strip_copy_u(&R.u[(ja + q) & 3][lane], u, nx, ny, ja + q, a, inner);
-      if constexpr (KIND == kRhsResidual) strip_copy_bn(&R.b[(ja + q - 1) & 3][lane], bn, nx, ny, ja + q - 1, a, lane_out);
+      if constexpr (kB) strip_copy_bn(&R.b[(ja + q - 1) & 3][lane], bn, nx, ny, ja + q - 1, a, lane_out);
       __pipeline_commit();
     }
     StripState s;
@@ -399,9 +440,9 @@ __global__ void __launch_bounds__(kST, 5)
       s.Lh = lh;
       s.Ll = ll;
       if (strip_fast(min(lo0, min(lo1, lo2)), max(hi0, max(hi1, hi2))))
-        strip_cells<true>(RK, Um1, Um2, Ua, lh, ll, rh, rl, s.lap, s.f0, s.f1);
+        strip_cells<true, KIND == kRhsReport>(RK, Um1, Um2, Ua, lh, ll, rh, rl, s.lap, s.f0, s.f1);
       else
-        strip_cells<false>(RK, Um1, Um2, Ua, lh, ll, rh, rl, s.lap, s.f0, s.f1);
+        strip_cells<false, KIND == kRhsReport>(RK, Um1, Um2, Ua, lh, ll, rh, rl, s.lap, s.f0, s.f1);
     }
     // row steps j = ja - 1 (state only) .. jb - 1; the state's rows j, j + 1
     // have ranges (lo1, hi1), (lo2, hi2).  Step j queues heights of row
@@ -410,22 +451,26 @@ __global__ void __launch_bounds__(kST, 5)
     for (int j = ja - 1; j < jb; ++j) {
       const bool out = j >= ja;
       strip_copy_u(&R.u[(j + 4) & 3][lane], u, nx, ny, j + 4, a, inner);
-      if constexpr (KIND == kRhsResidual) strip_copy_bn(&R.b[(j + 3) & 3][lane], bn, nx, ny, j + 3, a, lane_out);
+      if constexpr (kB) strip_copy_bn(&R.b[(j + 3) & 3][lane], bn, nx, ny, j + 3, a, lane_out);
       __pipeline_commit();
       __pipeline_wait_prior(2);
       df2 B = d2(p_splat(1.0f), p_splat(0.0f));
-      if constexpr (KIND == kRhsResidual) {
+      if constexpr (kB) {
         if (out) {
           const float4 v = R.b[j & 3][lane];
           B = d2(make_float2(v.x, v.z), make_float2(v.y, v.w));
         }
       }
-      const df2 U2 = strip_conv(R.u[(j + 2) & 3][lane], lo3, hi3);
+      const double2 v2 = R.u[(j + 2) & 3][lane];
+      const df2 U2 = strip_conv(v2, lo3, hi3);
+      if constexpr (KIND == kRhsReport) {
+        if (j + 2 > ja && j + 2 < jb) stats(v2);
+      }
       float gj;
       if (strip_fast(min(lo1, min(lo2, lo3)), max(hi1, max(hi2, hi3))))
-        gj = strip_step<KIND, true>(s, U2, B, out, j, a, lane_out, RK, nx, ny, bn, rhs, ulp);
+        gj = strip_step<KIND, true>(s, U2, B, out, j, a, lane_out, RK, nx, ny, bn, rhs, ulp, Gout, gmax);
       else
-        gj = strip_step<KIND, false>(s, U2, B, out, j, a, lane_out, RK, nx, ny, bn, rhs, ulp);
+        gj = strip_step<KIND, false>(s, U2, B, out, j, a, lane_out, RK, nx, ny, bn, rhs, ulp, Gout, gmax);
       if (!(gj <= g)) g = gj;
       lo1 = lo2;
       hi1 = hi2;
@@ -435,6 +480,49 @@ __global__ void __launch_bounds__(kST, 5)
     __pipeline_wait_prior(0);  // no copy outlives the warp
   }
   if constexpr (KIND == kRhsExplicit) return;
+  if constexpr (KIND == kRhsReport) {
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long g2 = __shfl_xor_sync(0xffffffffu, gmax, o), h2 = __shfl_xor_sync(0xffffffffu, hmin, o);
+      if (g2 > gmax) gmax = g2;
+      if (h2 < hmin) hmin = h2;
+      Mass128 m2;
+      m2.lo = __shfl_xor_sync(0xffffffffu, mass.lo, o);
+      m2.hi = __shfl_xor_sync(0xffffffffu, mass.hi, o);
+      mass_add(mass, m2);
+      nf |= __shfl_xor_sync(0xffffffffu, nf, o);
+    }
+    __shared__ unsigned long long sg[kSWarps], sh[kSWarps];
+    __shared__ Mass128 sm[kSWarps];
+    __shared__ int sn[kSWarps];
+    if (lane == 0) {
+      sg[warp] = gmax;
+      sh[warp] = hmin;
+      sm[warp] = mass;
+      sn[warp] = nf;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int k = 1; k < kSWarps; ++k) {
+        if (sg[k] > gmax) gmax = sg[k];
+        if (sh[k] < hmin) hmin = sh[k];
+        mass_add(mass, sm[k]);
+        nf |= sn[k];
+      }
+      PartX p;
+      p.gnorm = __longlong_as_double((long long)gmax);
+      p.pivot = 0;
+      p.pad = 0;
+      part[blockIdx.x] = p;
+      PartY q;
+      q.err = 0.0;
+      q.hmin = __longlong_as_double((long long)hmin);
+      q.mass = mass;
+      q.nonfinite = nf;
+      q.pivot = 0;
+      party[blockIdx.x] = q;
+    }
+    return;
+  }
   for (int o = 16; o > 0; o >>= 1) {
     const float g2 = __shfl_xor_sync(0xffffffffu, g, o);
     if (!(g2 <= g)) g = g2;
