@@ -31,12 +31,11 @@ int cuda_fail(cudaError_t e) { return e == cudaErrorMemoryAllocation ? TF_ERR_NO
   } while (0)
 
 
-// Reduce the partials of the last passes into the pinned c.hsc: the launch
-// and the copy are queued on the context's stream; finalize() also waits.
+// Reduce the partials of the last passes into the pinned c.hsc, queued on the
+// context's stream; finalize() also waits.
 int finalize_async(tf_ctx& c, int n_px, int n_py) {
-  tf::k_finalize<<<1, 256, 0, c.stream>>>(c.px, n_px, c.py, n_py, c.dsc);
+  tf::k_finalize<<<1, 256, 0, c.stream>>>(c.px, n_px, c.py, n_py, c.hsc);
   TF_CK(cudaGetLastError());
-  TF_CK(cudaMemcpyAsync(c.hsc, c.dsc, sizeof(Scalars), cudaMemcpyDeviceToHost, c.stream));
   return TF_OK;
 }
 // The same after an iteration of the partitioned path: the residual's
@@ -64,8 +63,8 @@ float elapsed(cudaEvent_t a, cudaEvent_t b) {
 // stream; iterate_collect() reads the result once the stream has reached it.
 // rhs_ready: the residual of this iteration was formed with b^n (the first
 // iteration of a step, explicit_launch with rhs0).
-int iterate_launch(tf_ctx& c, const double* u_k, double dt, double* u_next, double* w_out,
-                   double* v_out, bool rhs_ready = false) {
+int iterate_passes(tf_ctx& c, const double* u_k, double dt, double* u_next, double* w_out, double* v_out,
+                   bool rhs_ready) {
   const bool tm = c.timing.enabled;
   c.rhs_fused = rhs_ready;
   if (tm) TF_CK(cudaEventRecord(c.ev[0], c.stream));
@@ -77,6 +76,12 @@ int iterate_launch(tf_ctx& c, const double* u_k, double dt, double* u_next, doub
   if (tm) TF_CK(cudaEventRecord(c.ev[3], c.stream));
   TF_CK(c.ops->ysweep(c, u_k, dt, u_next, v_out));
   if (tm) TF_CK(cudaEventRecord(c.ev[4], c.stream));
+  return TF_OK;
+}
+int iterate_launch(tf_ctx& c, const double* u_k, double dt, double* u_next, double* w_out,
+                   double* v_out, bool rhs_ready = false) {
+  const int r = iterate_passes(c, u_k, dt, u_next, w_out, v_out, rhs_ready);
+  if (r) return r;
   return c.part ? finalize_part_async(c) : finalize_async(c, c.n_rhs_parts + c.grid_x, c.grid_y);
 }
 void iterate_collect(tf_ctx& c, bool w_out, Scalars* s) {
@@ -141,13 +146,8 @@ int film_stats(tf_ctx& c, const double* h, Scalars* s) {
   return TF_OK;
 }
 
-// Outcome of an iteration, in the oracle's order: pivot, positivity, test.
 int classify(const tf_ctx& c, const Scalars& s, int it, int fixed_iter) {
-  if (s.pivot) return TF_STEP_ZERO_PIVOT;
-  if (s.nonfinite) return TF_STEP_NONPOSITIVE;
-  if (fixed_iter > 0) return it >= fixed_iter ? TF_STEP_CONVERGED : TF_STEP_NOT_CONVERGED;
-  if (s.err < c.p.newton_tol) return TF_STEP_CONVERGED;
-  return TF_STEP_NOT_CONVERGED;
+  return tf::classify_iteration(s, it, fixed_iter, c.p.newton_tol);
 }
 
 void fill_info(tf_step_info* info, int status, int it, const Scalars& s) {
@@ -171,11 +171,45 @@ int step(tf_ctx& c, const double* h_old, double* h_new, double dt, int fixed_ite
   Scalars s;
   memset(&s, 0, sizeof(s));
   int status = TF_STEP_NOT_CONVERGED, it = 0;
+  // Iteration k + 1 is queued before the host reads the result of iteration
+  // k, so that the GPU never waits for the host: on a 64^2 film the round trip
+  // and the launches were a third of an iteration.  The device applies the
+  // same test, and what was queued behind the step's last iteration returns
+  // at once.  (Not with timing on, whose events serve one iteration, nor on
+  // the partitioned path.)
+  const bool ahead = !c.timing.enabled && !c.part;
+  auto queue = [&](int k) -> int {
+    c.ahead.mark = c.mark;
+    c.ahead.step = c.step_no;
+    int r = iterate_passes(c, k ? bufs[(k - 1) & 1] : h_old, dt, bufs[k & 1], nullptr, nullptr, k == 0);
+    const tf::RunAhead ra = c.ahead;
+    c.ahead = tf::RunAhead{nullptr, 0};
+    if (r) return r;
+    tf::k_iteration_end<<<1, 256, 0, c.stream>>>(c.px, c.n_rhs_parts + c.grid_x, c.py, c.grid_y, c.hsc + 1 + (k & 1), ra,
+                                                 c.mark, k + 1, fixed_iter, c.p.newton_tol);
+    TF_CK(cudaGetLastError());
+    TF_CK(cudaEventRecord(c.it_ev[k & 1], c.stream));
+    return TF_OK;
+  };
+  if (ahead) {
+    ++c.step_no;
+    const int r = queue(0);
+    if (r) return r;
+  }
   for (int k = 0; k < kmax; ++k) {
     double* un = bufs[k & 1];
-    int r = iterate(c, uk, dt, un, nullptr, nullptr, &s, k == 0);
-    if (r) return r;
-    if (k == 0) explicit_collect(c);
+    if (ahead) {
+      if (k + 1 < kmax) {
+        const int r = queue(k + 1);
+        if (r) return r;
+      }
+      TF_CK(cudaEventSynchronize(c.it_ev[k & 1]));
+      s = c.hsc[1 + (k & 1)];
+    } else {
+      const int r = iterate(c, uk, dt, un, nullptr, nullptr, &s, k == 0);
+      if (r) return r;
+      if (k == 0) explicit_collect(c);
+    }
     it = k + 1;
     uk = un;
     status = classify(c, s, it, fixed_iter);
@@ -360,10 +394,10 @@ int sweep_lines(int n, int precision, bool general) {
 int shared_lines(long long lines) {
   return lines <= 8 * kSMs ? 4 : (lines <= 16 * kSMs ? 8 : (lines <= 80 * kSMs ? 16 : 32));
 }
-// The sweeps' block shape, at least `least` lines per block.  In FP32-bulk with
-// the out-of-line mobility models the shapes round differently, so there the
-// shape depends on the film alone.
-void set_lines(tf_ctx& c, int least) {
+// The sweeps' block shape, at least `least` lines per block, and the residual's
+// strips.  In FP32-bulk with the out-of-line mobility models the sweeps' shapes
+// round differently, so there the shape depends on the film alone.
+void set_shapes(tf_ctx& c, int least) {
   if (c.p.precision != TF_FP64 && !c.packed_rhs) least = 0;
   const bool general = !(c.mk.model == TF_MODEL_POWERLAW && c.mk.n == 3 && c.mk.m == 2);
   const int x = sweep_lines(c.p.ny, c.p.precision, general), y = sweep_lines(c.p.nx, c.p.precision, general);
@@ -371,6 +405,20 @@ void set_lines(tf_ctx& c, int least) {
   c.nly = y > least ? y : least;
   c.grid_x = (c.p.ny + c.nlx - 1) / c.nlx;
   c.grid_y = (c.p.nx + c.nly - 1) / c.nly;
+  // residual strips: segments of 64 rows, halved (down to 16) until the grid
+  // holds two waves of warps (about 24 resident per SM), and, for a film alone,
+  // further (down to 2) while it still fits in one (20 per SM): a row step takes
+  // a warp about a microsecond, so a small film's residual is as long as its
+  // segments (64^2: 17 us in segments of 16 rows, 10 in segments of 2)
+  const long strips = (c.p.nx + tf::kRhsStripCols - 1) / tf::kRhsStripCols;
+  int rows = 64;
+  auto warps_at = [&](int r) { return strips * ((c.p.ny + r - 1) / r); };
+  while (rows > 16 && warps_at(rows) < 2L * kSMs * 24) rows /= 2;
+  while (least <= 4 && rows > 2 && rows <= 16 && warps_at(rows / 2) <= (long)kSMs * 20) rows /= 2;
+  c.strip_n = (int)strips;
+  c.strip_rows = rows;
+  c.grid_pkx = (int)((warps_at(rows) + tf::kRhsStripWarps - 1) / tf::kRhsStripWarps);
+  c.n_rhs_parts = c.packed_rhs ? c.grid_pkx : c.grid_rx * c.grid_ry;
 }
 // Films that advance at once run in blocks of at least shared_lines() lines;
 // their contexts go back to the shapes of a film alone afterwards.
@@ -380,10 +428,10 @@ struct SharedLines {
   SharedLines(int n_, tf_ctx* const* c) : n(n_), ctx(c) {
     long long lines = 0;
     for (int i = 0; i < n; ++i) lines += ctx[i]->p.nx > ctx[i]->p.ny ? ctx[i]->p.nx : ctx[i]->p.ny;
-    for (int i = 0; i < n; ++i) set_lines(*ctx[i], shared_lines(lines));
+    for (int i = 0; i < n; ++i) set_shapes(*ctx[i], shared_lines(lines));
   }
   ~SharedLines() {
-    for (int i = 0; i < n; ++i) set_lines(*ctx[i], 0);
+    for (int i = 0; i < n; ++i) set_shapes(*ctx[i], 0);
   }
 };
 
@@ -489,6 +537,9 @@ void tf_destroy(tf_ctx* c) {
   cudaFree(c->px);
   cudaFree(c->py);
   cudaFree(c->dsc);
+  cudaFree(c->mark);
+  for (int k = 0; k < 2; ++k)
+    if (c->it_ev[k]) cudaEventDestroy(c->it_ev[k]);
   if (c->hsc) cudaFreeHost(c->hsc);
   if (c->ens_exec) cudaGraphExecDestroy(c->ens_exec);
   cudaFree(c->ens_dev);
@@ -565,25 +616,8 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
   mk.pol_d = p->pol_d;
   c->grid_rx = (p->nx + 31) / 32;
   c->grid_ry = (p->ny + 31) / 32;
-  {
-    // residual strips: segments of 64 rows, halved (down to 16) until the
-    // grid holds two waves of warps (about 24 resident per SM), and further
-    // (down to 2) while it still fits in one (20 per SM): a row step takes a
-    // warp about a microsecond, so a small film's residual is as long as its
-    // segments (64^2: 17 us in segments of 16 rows)
-    const long strips = (p->nx + tf::kRhsStripCols - 1) / tf::kRhsStripCols;
-    int rows = 64;
-    auto warps_at = [&](int r) { return strips * ((p->ny + r - 1) / r); };
-    while (rows > 16 && warps_at(rows) < 2L * kSMs * 24) rows /= 2;
-    while (rows > 2 && rows <= 16 && warps_at(rows / 2) <= (long)kSMs * 20) rows /= 2;
-    const long warps = strips * ((p->ny + rows - 1) / rows);
-    c->strip_n = (int)strips;
-    c->strip_rows = rows;
-    c->grid_pkx = (int)((warps + tf::kRhsStripWarps - 1) / tf::kRhsStripWarps);
-  }
   c->packed_rhs = p->precision != TF_FP64 && p->model == TF_MODEL_POWERLAW && p->n == 3 && p->m == 2;
-  set_lines(*c, 0);
-  c->n_rhs_parts = c->packed_rhs ? c->grid_pkx : c->grid_rx * c->grid_ry;
+  set_shapes(*c, 0);
   c->grid_st_x = (p->nx + 15) / 16;
   c->grid_st_y = (p->ny + 15) / 16;
   c->grid_stats = 1216;  // 8 blocks of 256 threads per SM on 152 SMs
@@ -632,7 +666,13 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
   if (!r) r = dalloc(&c->py, (size_t)c->n_py * sizeof(tf::PartY));
   if (!r) r = dalloc(&c->dsc, sizeof(Scalars));
   if (!r) {
-    e = cudaMallocHost((void**)&c->hsc, sizeof(Scalars));
+    e = cudaMallocHost((void**)&c->hsc, 3 * sizeof(Scalars));
+    if (e != cudaSuccess) r = cuda_fail(e);
+  }
+  if (!r) r = dalloc(&c->mark, sizeof(int));
+  if (!r && cudaMemset(c->mark, 0, sizeof(int)) != cudaSuccess) r = TF_ERR_CUDA;
+  for (int k = 0; k < 2 && !r; ++k) {
+    e = cudaEventCreateWithFlags(&c->it_ev[k], cudaEventDisableTiming);
     if (e != cudaSuccess) r = cuda_fail(e);
   }
   for (int k = 0; k < 8 && !r; ++k) {
@@ -776,7 +816,7 @@ int tf_advance(tf_ctx* c, double* h, double t0, double t_end, double dt0, int ma
 bool graph_capable(const tf_ctx& c) { return c.ops->ens_graph && c.packed_rhs && !c.part; }
 
 int film_graph_start(tf_ctx& c, double* h, double t0, double t_end, double dt0, int max_att, int streak) {
-  if (c.ens_exec && (c.ens_nlx != c.nlx || c.ens_nly != c.nly)) {  // built for other block shapes
+  if (c.ens_exec && (c.ens_nlx != c.nlx || c.ens_nly != c.nly || c.ens_rows != c.strip_rows)) {  // built for other shapes
     TF_CK(cudaGraphExecDestroy(c.ens_exec));
     c.ens_exec = nullptr;
   }
@@ -789,6 +829,7 @@ int film_graph_start(tf_ctx& c, double* h, double t0, double t_end, double dt0, 
     TF_CK(c.ops->ens_graph(c, c.ens_dev, &c.ens_exec));
     c.ens_nlx = c.nlx;
     c.ens_nly = c.nly;
+    c.ens_rows = c.strip_rows;
   }
   tf::EnsDev& e = *c.ens_host;
   memset(&e, 0, sizeof(e));
@@ -972,7 +1013,7 @@ int tf_tune_line_solver(const tf_params* p, void* stream, const double* h, doubl
         break;
       }
       rc = tf_init(&q, st[(size_t)k], &ctx[(size_t)k]);
-      if (!rc) set_lines(*ctx[(size_t)k], shared_lines((long long)copies * (q.nx > q.ny ? q.nx : q.ny)));
+      if (!rc) set_shapes(*ctx[(size_t)k], shared_lines((long long)copies * (q.nx > q.ny ? q.nx : q.ny)));
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!rc && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) rc = TF_ERR_CUDA;

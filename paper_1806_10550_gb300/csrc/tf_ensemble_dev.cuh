@@ -46,14 +46,6 @@ struct EnsDev {
   unsigned long long kernels;  // kernel launches the graph ran for this film
 };
 
-TF_HD int ens_classify(const Scalars& s, int it, int fixed_iter, double tol) {
-  if (s.pivot) return TF_STEP_ZERO_PIVOT;
-  if (s.nonfinite) return TF_STEP_NONPOSITIVE;
-  if (fixed_iter > 0) return it >= fixed_iter ? TF_STEP_CONVERGED : TF_STEP_NOT_CONVERGED;
-  if (s.err < tol) return TF_STEP_CONVERGED;
-  return TF_STEP_NOT_CONVERGED;
-}
-
 // Start the next attempt: false when the film is done (attempt budget spent
 // or t_end reached).  The step's Δt is clipped to land on t_end.
 __device__ __forceinline__ bool ens_start_attempt(EnsDev& e) {
@@ -102,14 +94,14 @@ static __global__ void k_ens_begin(EnsDev* __restrict__ e, cudaGraphConditionalH
 // other iterate buffer) or end the step.
 static __global__ void __launch_bounds__(256)
     k_ens_iter(const PartX* __restrict__ px, int nx_part, const PartY* __restrict__ py, int ny_part,
-               Scalars* __restrict__ out, EnsDev* __restrict__ e, cudaGraphConditionalHandle inner) {
-  if (!finalize_block(px, nx_part, py, ny_part, out)) return;
+               EnsDev* __restrict__ e, cudaGraphConditionalHandle inner) {
+  Scalars s;
+  if (!finalize_block(px, nx_part, py, ny_part, s)) return;
   EnsDev& E = *e;
-  const Scalars s = *out;
   E.kernels += E.k == 0 ? 3 : 4;
   E.it = E.k + 1;
   E.p.uk = E.p.un;
-  E.sstatus = ens_classify(s, E.it, E.fixed_iter, E.tol);
+  E.sstatus = classify_iteration(s, E.it, E.fixed_iter, E.tol);
   ++E.k;
   const bool more = E.sstatus == TF_STEP_NOT_CONVERGED && E.k < E.kmax;
   if (more) E.p.un = (E.k & 1) ? E.ubuf : E.p.nxt;
@@ -130,11 +122,10 @@ static __global__ void __launch_bounds__(256) k_ens_copy(const EnsDev* __restric
 // grow_after accepted steps in a row, rupture, Δt floor) and the next
 // attempt.
 static __global__ void __launch_bounds__(256)
-    k_ens_step(const PartY* __restrict__ py, int ny_part, Scalars* __restrict__ out, EnsDev* __restrict__ e,
-               cudaGraphConditionalHandle outer) {
-  if (!finalize_block(nullptr, 0, py, ny_part, out)) return;
+    k_ens_step(const PartY* __restrict__ py, int ny_part, EnsDev* __restrict__ e, cudaGraphConditionalHandle outer) {
+  Scalars s;
+  if (!finalize_block(nullptr, 0, py, ny_part, s)) return;
   EnsDev& E = *e;
-  const Scalars* s = out;
   E.kernels += 4;
   ++E.a;
   E.newton_iterations += E.it;
@@ -149,7 +140,7 @@ static __global__ void __launch_bounds__(256)
       E.dt = fmin(E.dt * E.dt_grow, E.dt_max);
       E.streak = 0;
     }
-    if (E.rupture_h > 0.0 && s->hmin < E.rupture_h) {
+    if (E.rupture_h > 0.0 && s.hmin < E.rupture_h) {
       E.status = TF_ADV_RUPTURE;
       E.done = 1;
     } else {

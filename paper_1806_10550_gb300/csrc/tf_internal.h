@@ -117,7 +117,11 @@ struct tf_ctx {
   tf::PartY* py;
   int n_px, n_py;
   tf::Scalars* dsc;
-  tf::Scalars* hsc;  // pinned
+  tf::Scalars* hsc;  // pinned, 3: the last reduction's; two iterations in flight (see step())
+  tf::RunAhead ahead;  // of the iteration being queued
+  int* mark;         // RunAhead's mark
+  int step_no;       // number of the step in flight
+  cudaEvent_t it_ev[2];  // ends of the two iterations in flight
   tf_timing timing;
   cudaEvent_t ev[8];  // 0-4 iteration timing, 5-6 explicit-part timing, 7 work done (ensembles)
   bool rhs_fused;     // the iteration in flight had its residual formed with b^n
@@ -128,5 +132,5 @@ struct tf_ctx {
   tf::EnsDev* ens_dev;        // the film's device-resident controller state
   tf::EnsDev* ens_host;       // pinned staging copy of it
   cudaGraphExec_t ens_exec;   // the instantiated graph of a whole run
-  int ens_nlx, ens_nly;       // the lines per sweep block it was built with
+  int ens_nlx, ens_nly, ens_rows;  // the lines per sweep block and rows per strip segment it was built with
 };

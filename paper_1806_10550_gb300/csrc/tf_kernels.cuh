@@ -25,6 +25,7 @@
 
 #include <cuda_runtime.h>
 
+#include "../../include/tf.h"
 #include "tf_numeric.cuh"
 
 namespace tf {
@@ -641,64 +642,95 @@ __device__ __forceinline__ bool positive_finite_bits(double u) {
 // Reductions over the per-block partials (one block, fixed order).
 
 // The reduction of the per-block partials into the iteration's scalars by
-// one block of 256 threads: thread 0 writes *out and returns true.
+// one block of 256 threads: true in thread 0, which has them in s.  Values of
+// a warp meet by shuffles and the eight warps' in one step, without a tree of
+// block barriers.
+__device__ __forceinline__ void scalars_join(Scalars& a, const Scalars& b) {
+  if (!(b.err <= a.err)) a.err = b.err;
+  if (!(b.gnorm <= a.gnorm)) a.gnorm = b.gnorm;
+  a.hmin = fmin(a.hmin, b.hmin);
+  mass_add(a.mass, b.mass);
+  a.nonfinite |= b.nonfinite;
+  a.pivot |= b.pivot;
+}
 __device__ __forceinline__ bool finalize_block(const PartX* __restrict__ px, int nx_part,
-                                               const PartY* __restrict__ py, int ny_part,
-                                               Scalars* __restrict__ out) {
-  __shared__ double s_err[256], s_g[256], s_h[256];
-  __shared__ Mass128 s_m[256];
-  __shared__ int s_nf[256], s_pv[256];
+                                               const PartY* __restrict__ py, int ny_part, Scalars& s) {
+  __shared__ Scalars sw[8];
   const int t = threadIdx.x;
-  double err = 0.0, g = 0.0, h = INFINITY;
-  Mass128 m = {0ull, 0ull};
-  int nf = 0, pv = 0;
+  s.err = s.gnorm = 0.0;
+  s.hmin = INFINITY;
+  s.mass.lo = s.mass.hi = 0ull;
+  s.nonfinite = s.pivot = 0;
+#pragma unroll 4
   for (int k = t; k < nx_part; k += 256) {
-    if (!(px[k].gnorm <= g)) g = px[k].gnorm;
-    pv |= px[k].pivot;
+    const double g = px[k].gnorm;
+    if (!(g <= s.gnorm)) s.gnorm = g;
+    s.pivot |= px[k].pivot;
   }
+#pragma unroll 2
   for (int k = t; k < ny_part; k += 256) {
-    if (!(py[k].err <= err)) err = py[k].err;
-    h = fmin(h, py[k].hmin);
-    mass_add(m, py[k].mass);
-    nf |= py[k].nonfinite;
-    pv |= py[k].pivot;
+    const PartY p = py[k];
+    if (!(p.err <= s.err)) s.err = p.err;
+    s.hmin = fmin(s.hmin, p.hmin);
+    mass_add(s.mass, p.mass);
+    s.nonfinite |= p.nonfinite;
+    s.pivot |= p.pivot;
   }
-  s_err[t] = err;
-  s_g[t] = g;
-  s_h[t] = h;
-  s_m[t] = m;
-  s_nf[t] = nf;
-  s_pv[t] = pv;
+  for (int o = 16; o > 0; o >>= 1) {
+    Scalars b;
+    b.err = __shfl_down_sync(0xffffffffu, s.err, o);
+    b.gnorm = __shfl_down_sync(0xffffffffu, s.gnorm, o);
+    b.hmin = __shfl_down_sync(0xffffffffu, s.hmin, o);
+    b.mass.lo = __shfl_down_sync(0xffffffffu, s.mass.lo, o);
+    b.mass.hi = __shfl_down_sync(0xffffffffu, s.mass.hi, o);
+    b.nonfinite = __shfl_down_sync(0xffffffffu, s.nonfinite, o);
+    b.pivot = __shfl_down_sync(0xffffffffu, s.pivot, o);
+    if ((t & 31) + o < 32) scalars_join(s, b);
+  }
+  if ((t & 31) == 0) sw[t >> 5] = s;
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (t < o) {
-      if (!(s_err[t + o] <= s_err[t])) s_err[t] = s_err[t + o];
-      if (!(s_g[t + o] <= s_g[t])) s_g[t] = s_g[t + o];
-      s_h[t] = fmin(s_h[t], s_h[t + o]);
-      mass_add(s_m[t], s_m[t + o]);
-      s_nf[t] |= s_nf[t + o];
-      s_pv[t] |= s_pv[t + o];
-    }
-    __syncthreads();
-  }
-  if (t == 0) {
-    Scalars s;
-    s.err = s_err[0];
-    s.gnorm = s_g[0];
-    s.hmin = s_h[0];
-    s.mass = s_m[0];
-    s.nonfinite = s_nf[0];
-    s.pivot = s_pv[0];
-    *out = s;
-    return true;
-  }
-  return false;
+  if (t != 0) return false;
+  for (int k = 1; k < 8; ++k) scalars_join(s, sw[k]);
+  return true;
 }
 
+// out: device memory, or pinned host memory (the host reads it once the
+// stream has passed this kernel; no copy is queued).
 static __global__ void __launch_bounds__(256)
     k_finalize(const PartX* __restrict__ px, int nx_part, const PartY* __restrict__ py, int ny_part,
                Scalars* __restrict__ out) {
-  finalize_block(px, nx_part, py, ny_part, out);
+  Scalars s;
+  if (finalize_block(px, nx_part, py, ny_part, s)) *out = s;
+}
+
+// A step's iterations are queued one ahead of the host's reading of their
+// results: the kernels of an iteration that follows the step's last return
+// at once.  *mark == step says that step number `step` has ended; mark NULL
+// where nothing runs ahead.
+struct RunAhead {
+  const int* mark;
+  int step;
+  __device__ __forceinline__ bool over() const { return mark && *mark == step; }
+};
+
+// Outcome of an iteration, in the oracle's order: pivot, positivity, test.
+TF_HD int classify_iteration(const Scalars& s, int it, int fixed_iter, double tol) {
+  if (s.pivot) return TF_STEP_ZERO_PIVOT;
+  if (s.nonfinite) return TF_STEP_NONPOSITIVE;
+  if (fixed_iter > 0) return it >= fixed_iter ? TF_STEP_CONVERGED : TF_STEP_NOT_CONVERGED;
+  if (s.err < tol) return TF_STEP_CONVERGED;
+  return TF_STEP_NOT_CONVERGED;
+}
+// The end of iteration `it` (from 1): its scalars to the host, and the step's
+// mark when it is the last.
+static __global__ void __launch_bounds__(256)
+    k_iteration_end(const PartX* __restrict__ px, int nx_part, const PartY* __restrict__ py, int ny_part,
+                    Scalars* __restrict__ out, RunAhead ra, int* mark, int it, int fixed_iter, double tol) {
+  if (ra.over()) return;
+  Scalars s;
+  if (!finalize_block(px, nx_part, py, ny_part, s)) return;
+  *out = s;
+  if (classify_iteration(s, it, fixed_iter, tol) != TF_STEP_NOT_CONVERGED) *mark = ra.step;
 }
 
 // Mass and minimum of a grid (for tf_residual's norms).

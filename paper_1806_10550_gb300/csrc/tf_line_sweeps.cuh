@@ -370,8 +370,9 @@ __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
     k_ysweep(ModelK M, LineK<typename Mode::LP> Lp, const double* __restrict__ up,
              const typename Mode::LP* __restrict__ ul, const typename Mode::LP* __restrict__ w,
              typename Mode::LP* __restrict__ fac, double* __restrict__ unp, double* __restrict__ vout,
-             PartY* __restrict__ part, const LineK<typename Mode::LP>* __restrict__ Ld = nullptr,
-             const double* const* __restrict__ uio = nullptr) {
+             PartY* __restrict__ part, const LineK<typename Mode::LP>* __restrict__ Ld,
+             const double* const* __restrict__ uio, RunAhead ra) {
+  if (ra.over()) return;
   typedef typename Mode::LP LP;
   const LineK<LP>& L = DEV ? *Ld : Lp;
   const double* __restrict__ u = DEV ? uio[0] : up;
@@ -648,7 +649,8 @@ template <class Mode, bool DEV, bool GEN>
 __global__ void __launch_bounds__(kSweepThreads, Mode::kSweepBlocks)
     k_xsweep(ModelK M, LineK<typename Mode::LP> Lp, const typename Mode::LP* __restrict__ ul,
              typename Mode::LP* __restrict__ rw, typename Mode::LP* __restrict__ fac,
-             PartX* __restrict__ part, const LineK<typename Mode::LP>* __restrict__ Ld = nullptr) {
+             PartX* __restrict__ part, const LineK<typename Mode::LP>* __restrict__ Ld, RunAhead ra) {
+  if (ra.over()) return;
   typedef typename Mode::LP LP;
   const LineK<LP>& L = DEV ? *Ld : Lp;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -28,13 +28,13 @@ template <class Mode> struct Launch {
   template <int NL, bool DEV, bool GEN>
   static void narrow_x(tf_ctx& c, const LineK<LP>& L, const LP* ul, const LineK<LP>* Ld, cudaStream_t s) {
     k_narrow_sweep<Mode, NL, 0, DEV, GEN><<<c.grid_x, NarrowCfg<LP, NL>::NT, smem_n<NL, 0>, s>>>(
-        c.mk, L, nullptr, ul, (LP*)c.w, (LP*)c.fac_x, nullptr, nullptr, c.px + c.n_rhs_parts, nullptr, Ld, nullptr);
+        c.mk, L, nullptr, ul, (LP*)c.w, (LP*)c.fac_x, nullptr, nullptr, c.px + c.n_rhs_parts, nullptr, Ld, nullptr, c.ahead);
   }
   template <int NL, bool DEV, bool GEN>
   static void narrow_y(tf_ctx& c, const LineK<LP>& L, const double* u, const LP* ul, double* un, double* v,
                        const LineK<LP>* Ld, const double* const* uio, cudaStream_t s) {
     k_narrow_sweep<Mode, NL, 1, DEV, GEN><<<c.grid_y, NarrowCfg<LP, NL>::NT, smem_n<NL, 1>, s>>>(
-        c.mk, L, u, ul, (LP*)c.w, (LP*)c.fac_y, un, v, nullptr, c.py, Ld, uio);
+        c.mk, L, u, ul, (LP*)c.w, (LP*)c.fac_y, un, v, nullptr, c.py, Ld, uio, c.ahead);
   }
   template <bool DEV, bool GEN>
   static void launch_x(tf_ctx& c, const LineK<LP>& L, const LP* ul, const LineK<LP>* Ld, cudaStream_t s) {
@@ -45,7 +45,7 @@ template <class Mode> struct Launch {
       default:
         if constexpr (kWide<GEN>)
           k_xsweep<Mode, DEV, GEN><<<c.grid_x, kSweepThreads, smem_x, s>>>(c.mk, L, ul, (LP*)c.w, (LP*)c.fac_x,
-                                                                         c.px + c.n_rhs_parts, Ld);
+                                                                         c.px + c.n_rhs_parts, Ld, c.ahead);
     }
   }
   template <bool DEV, bool GEN>
@@ -58,7 +58,7 @@ template <class Mode> struct Launch {
       default:
         if constexpr (kWide<GEN>)
           k_ysweep<Mode, DEV, GEN><<<c.grid_y, kSweepThreads, smem_y, s>>>(c.mk, L, u, ul, (const LP*)c.w, (LP*)c.fac_y,
-                                                                         un, v, c.py, Ld, uio);
+                                                                         un, v, c.py, Ld, uio, c.ahead);
     }
   }
   // Dynamic shared memory of a sweep kernel; two blocks share an SM only with
@@ -143,14 +143,15 @@ template <class Mode> struct Launch {
     if constexpr (kF32B) {
       if (c.packed_rhs) {
         k_rhs_strip<kRhsResidual><<<c.grid_pkx, kST, 0, c.stream>>>(
-            c.mk, strip_consts(c.mk, step(c, dt), false), u_k, (HP*)c.bn, (LP*)c.w, (LP*)c.ulp, c.px, c.strip_n, c.strip_rows);
+            c.mk, strip_consts(c.mk, step(c, dt), false), u_k, (HP*)c.bn, (LP*)c.w, (LP*)c.ulp, c.px, c.strip_n, c.strip_rows,
+            nullptr, nullptr, nullptr, nullptr, c.ahead);
         return cudaGetLastError();
       }
     }
     dim3 grid(c.grid_rx, c.grid_ry);
     k_rhs<Mode, kRhsResidual><<<grid, 256, smem_rhs, c.stream>>>(c.mk, rhs_consts<HP>(c.mk, step(c, dt)), u_k,
                                                    (HP*)c.bn, (LP*)c.w,
-                                                   (LP*)c.ulp, c.px);
+                                                   (LP*)c.ulp, c.px, c.ahead);
     return cudaGetLastError();
   }
   // b^n of a step and the right side of its first iteration (u_0 = u^n)
@@ -231,7 +232,7 @@ template <class Mode> struct Launch {
       auto sweeps = [&]() {
         launch_x<true, false>(c, l0, (const LP*)c.ulp, &e->line, s);
         launch_y<true, false>(c, l0, nullptr, (const LP*)c.ulp, nullptr, nullptr, &e->line, &e->p.uk, s);
-        k_ens_iter<<<1, 256, 0, s>>>(c.px, c.n_rhs_parts + c.grid_x, c.py, c.grid_y, c.dsc, e, hi);
+        k_ens_iter<<<1, 256, 0, s>>>(c.px, c.n_rhs_parts + c.grid_x, c.py, c.grid_y, e, hi);
       };
       if ((err = cudaGraphCreate(&g, 0))) return fail(err);
       if ((err = cudaGraphConditionalHandleCreate(&ho, g, 0, cudaGraphCondAssignDefault))) return fail(err);
@@ -283,7 +284,7 @@ template <class Mode> struct Launch {
       if ((err = cudaStreamBeginCaptureToGraph(s, B, &ni, nullptr, 1, md))) return fail(err);
       k_ens_copy<<<1024, 256, 0, s>>>(e, c.N);
       k_grid_stats<<<c.grid_stats, 256, 0, s>>>(nullptr, c.N, c.py, &e->p.nxt);
-      k_ens_step<<<1, 256, 0, s>>>(c.py, c.grid_stats, c.dsc, e, ho);
+      k_ens_step<<<1, 256, 0, s>>>(c.py, c.grid_stats, e, ho);
       if ((err = cudaStreamEndCapture(s, &B))) return fail(err);
       cudaGraphExec_t x = nullptr;  // *out only ever holds an instantiated graph
       if ((err = cudaGraphInstantiate(&x, g, 0))) return fail(err);

@@ -148,7 +148,8 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
                    const typename Mode::LP* __restrict__ ul, typename Mode::LP* w, typename Mode::LP* __restrict__ fac,
                    double* __restrict__ unp, double* __restrict__ vout, PartX* __restrict__ partx,
                    PartY* __restrict__ party, const LineK<typename Mode::LP>* __restrict__ Ld,
-                   const double* const* __restrict__ uio) {
+                   const double* const* __restrict__ uio, RunAhead ra) {
+  if (ra.over()) return;
   typedef typename Mode::LP LP;
   typedef NarrowCfg<LP, NL> Cf;
   constexpr int C = Cf::C, G = Cf::G, D = Cf::D, R = Cf::R, NP = Cf::NP;

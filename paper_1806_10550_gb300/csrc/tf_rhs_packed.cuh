@@ -385,7 +385,8 @@ __global__ void __launch_bounds__(kST, 5)
     k_rhs_strip(ModelK M, StripK RKp, const double* __restrict__ up, df64* __restrict__ bn,
                 float* __restrict__ rhs, float* __restrict__ ulp, PartX* __restrict__ part, int nstrip,
                 int seg_rows, const StripK* __restrict__ RKd = nullptr, const double* const* __restrict__ ud = nullptr,
-                double* __restrict__ Gout = nullptr, PartY* __restrict__ party = nullptr) {
+                double* __restrict__ Gout = nullptr, PartY* __restrict__ party = nullptr, RunAhead ra = {nullptr, 0}) {
+  if (ra.over()) return;
   constexpr bool kB = KIND == kRhsResidual || KIND == kRhsReport;  // reads b^n
   const StripK& RK = DEV ? *RKd : RKp;
   const double* __restrict__ u = DEV ? *ud : up;

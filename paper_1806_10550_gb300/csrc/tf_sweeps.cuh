@@ -64,7 +64,8 @@ __global__ void __launch_bounds__(256, 4)  // shared memory allows 4 blocks per 
     k_rhs(ModelK M, RhsK<typename Mode::HP> RK, const double* __restrict__ u,
           typename Mode::HP* __restrict__ bn,
           typename Mode::LP* __restrict__ rhs, typename Mode::LP* __restrict__ ul,
-          PartX* __restrict__ part) {
+          PartX* __restrict__ part, RunAhead ra = {nullptr, 0}) {
+  if (ra.over()) return;
   typedef typename Mode::HP HP;
   typedef typename Mode::LP LP;
   constexpr int T = 32, NT = 256;
