@@ -124,23 +124,17 @@ TF_HD float rcp(float x) {
   return 1.0f / x;
 #endif
 }
-// Reciprocal of the FP64 line solves and of the FP64 Jacobian's heights: a
-// float seed r0 of 1/x (relative error e = 1 - x r0 of about 2^-22, the
-// mantissas crossing between the formats with integer operations) and one
-// third-order step, 1/x = r0 (1 + e + e^2) + O(e^3): three FP64 operations,
+// Reciprocal of the FP64 line solves and of the FP64 Jacobian's heights: the
+// hardware's approximate reciprocal r0 (at least 2^-18 good: e = 1 - x r0) and
+// one third-order step, 1/x = r0 (1 + e + e^2) + O(e^3): three FP64 operations,
 // rounded once at the end.  What bounds the FP64 sweeps is the number of FP64
-// instructions (a warp's takes 64 cycles of its sub-partition's pipe whatever
+// instructions (a warp's takes 65 cycles of its sub-partition's pipe whatever
 // its lanes).  Zero, non-finite and extreme arguments take the division.
 __device__ __forceinline__ double rcp3(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned ex = (hi >> 20) & 0x7ffu;
-  if (ex - 64u > 1918u) return 1.0 / x;  // the seed and 1/x are normal for exponents 64 .. 1982
-  const float m = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));  // |x| / 2^(ex - 1023), truncated
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(m));  // in [1/2, 1]
-  const unsigned rb = __float_as_uint(r);
-  const double r0 =
-      __hiloint2double((int)(((rb >> 3) + ((896u + 1023u - ex) << 20)) | (hi & 0x80000000u)), (int)(rb << 29));
+  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (ex - 64u > 1918u) return 1.0 / x;  // r0 and 1/x are normal for exponents 64 .. 1982
+  double r0;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
   const double e = fma(-x, r0, 1.0);
   return fma(r0, fma(e, e, e), r0);
 }

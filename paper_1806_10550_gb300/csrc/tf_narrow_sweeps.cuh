@@ -6,21 +6,21 @@
 // its own, and the warps are placed by the SM sub-partition (warp index mod
 // 4) that they run on.
 //   warp 0            the recurrences of both halves of every line (lane =
-//                     half * NL + line), alone on its sub-partition but for
-//                     the loaders, which do no arithmetic
-//   loaders           every cp.async tile copy (FP64: warps 4 and 8)
+//                     half * NL + line)
+//   loaders           every cp.async tile copy
 //   the others        producers (band rows; update and reductions on the way
-//                     back) and, in FP64, one warp for the recurrence of the
-//                     right side
+//                     back) and, in FP64, two more warps of the elimination
 // FP64 on this chip is bound by instructions: a sub-partition takes 65 cycles
 // for a warp's FP64 instruction, however many lanes it carries (one warp's
 // dependent ones 71 to 87, four independent 263; with ten warps 19.5 cycles
 // an instruction over the SM).  One warp for both halves spends half of what
-// a warp per half does, and the right side's three operations a cell go to
-// another sub-partition: the recurrence warp is left with nine FP64
-// operations a cell where each of two warps had fifteen and shared its pipe
-// with producers.  1024^2, 8 lines a block: 890 cycles a cell against 1350,
-// sweeps 317/322 us against 422/430 (and 701/772 in blocks of 32).
+// a warp per half does.  The elimination's twelve operations a cell are three
+// warps': warp 0 forms the pivot, its inverse and g (five, the chain); warp 4,
+// beside it on sub-partition 0 where no producer runs, d and the next cells'
+// coefficients (four, while warp 0 inverts); and the right side (three) is
+// carried on another sub-partition, a few cells behind.  1024^2, 8 lines a
+// block: sweeps of 289/294 us; 317/322 with warp 0 doing nine (890 cycles a
+// cell), 422/430 with a warp per half doing fifteen beside producers (1350).
 // FP32: a tick is the recurrence's (52 cycles a cell) instead of the
 // producers' copies and band rows; 1024^2 37/45 us against 42/53 with copying
 // producers and 69/86 in blocks of 32.
@@ -42,7 +42,7 @@ template <class LP, int NL> struct NarrowCfg {
   // cycles (one warp took 1500 to 1950), an FP64 tick is ten times longer
   static constexpr int LW = Z ? (PW > 3 ? 2 : 1) : (PW > 3 ? 3 : 4);
   static constexpr int NLD = 32 * LW;              // loader threads
-  static constexpr int NW = 1 + LW + PW + (Z ? 1 : 0);
+  static constexpr int NW = 1 + LW + PW + (Z ? 2 : 0);
   static constexpr int NT = 32 * NW;
   static constexpr int D = 4, R = 5;               // ring slots, forward and backward tiles
   static constexpr int XP = 36;                    // row pitch of the x sweep's tiles (whole 16-byte vectors)
@@ -50,10 +50,23 @@ template <class LP, int NL> struct NarrowCfg {
   static constexpr int FH = 3 * C * NL + NL;       // a half's factors of a chunk, padded: the halves on different banks
   static constexpr int SUB = 6;                    // cells between two hand-overs to the right side's warp
   static_assert(PW * 32 == NP && PW % 3 == 0 && C % SUB == 0, "whole warps, three of four sub-partitions");
-  // roles of the warps after warp 0: FP64, loaders at the multiples of 4;
-  // FP32, the producers and then the loaders
-  __device__ static bool loader(int w) { return Z ? w != 0 && (w & 3) == 0 : w > PW; }
-  __device__ static int index(int w) { return Z ? ((w & 3) ? w - 1 - w / 4 : w / 4 - 1) : (w > PW ? w - 1 - PW : w - 1); }
+  // Roles of the warps, and a warp's index within its role.  FP32: warp 0, the
+  // producers, the loaders.  FP64: warps 0 and 4 (kCoef) on sub-partition 0,
+  // producers from 1 on, then the loaders and the right side's warp, none of
+  // them on sub-partition 0 but a loader, which has no arithmetic.
+  enum Role { kChain, kProducer, kCoef, kRight, kLoader };
+  __device__ static Role role(int w) {
+    if (w == 0) return kChain;
+    if (!Z) return w <= PW ? kProducer : kLoader;
+    if (w == 4) return kCoef;
+    if (w < 4 || (PW == 6 && w < 8)) return kProducer;
+    return w == (PW == 6 ? 9 : 5) ? kRight : kLoader;
+  }
+  __device__ static int index(int w) {
+    if (!Z) return w > PW ? w - 1 - PW : w - 1;
+    if (role(w) == kLoader) return PW == 6 ? (w - 8) / 2 : 0;
+    return w < 4 ? w - 1 : w - 2;  // producers
+  }
 };
 
 template <class LP, int NL, int DIR> struct NarrowFwd {
@@ -62,7 +75,10 @@ template <class LP, int NL, int DIR> struct NarrowFwd {
   LP ut[Cf::D][2][DIR == 0 ? (NL + 2) * Cf::XP : (Cf::C + 4) * Cf::YP];
   LP rt[Cf::D][2][DIR == 0 ? NL * Cf::XP : Cf::C * NL];  // right sides (x: [row][col], y: [row][col])
   LP band[2][6][Cf::C][2 * NL];                          // [stage][a..e, r][cell][half, line]
-  LP bi[Cf::Z ? Cf::C : 1][2 * NL][2];                   // beta and 1/mu for the right side's warp
+  // FP64, between the elimination's warps: beta and 1/mu of a chunk for the
+  // right side; 1/mu and g of a cell; beta, c - a d'' and d - beta d' of the next
+  LP bi[Cf::Z ? Cf::C : 1][2 * NL][2];
+  LP ig[2 * NL][2], co[2 * NL][5];
 };
 template <class LP, int NL, int DIR> struct NarrowBwd {
   typedef NarrowCfg<LP, NL> Cf;
@@ -80,11 +96,11 @@ template <class LP, int NL, int DIR> struct NarrowSmem {
   PartY part[NarrowCfg<LP, NL>::NW];
 };
 
-// A zero or non-finite pivot mu (inv = 1/mu) shows in bad, or as a NaN of chk.
-__device__ __forceinline__ void pivot_check(float mu, float inv, float& chk, int&) { chk = fma(mu, inv, chk); }
-__device__ __forceinline__ void pivot_check(double mu, double, double&, int& bad) {  // no FP64 operation
-  const unsigned hi = (unsigned)__double2hiint(mu) & 0x7fffffffu;
-  if (hi >= 0x7ff00000u || (hi | (unsigned)__double2loint(mu)) == 0u) bad = 1;
+// Whether the inverse of a pivot shows that the pivot is zero or not finite
+// (no FP64 operation).
+__device__ __forceinline__ bool zero_or_nonfinite(double inv) {
+  const unsigned hi = (unsigned)__double2hiint(inv) & 0x7fffffffu;
+  return hi >= 0x7ff00000u || (hi | (unsigned)__double2loint(inv)) == 0u;
 }
 
 // R x W tile columns [col0, col0 + W) x rows [row0, row0 + R) of a row-major
@@ -159,11 +175,10 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
   extern __shared__ __align__(16) unsigned char smem_raw[];
   NarrowSmem<LP, NL, DIR>& S = *reinterpret_cast<NarrowSmem<LP, NL, DIR>*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool chain = warp == 0, loader = Cf::loader(warp);
-  const int other = Cf::index(warp);  // index within the role
-  const bool zwarp = Cf::Z && !chain && !loader && other == Cf::PW;
-  const bool producer = !chain && !loader && !zwarp;
-  const int p = other * 32 + lane;
+  const typename Cf::Role role = Cf::role(warp);
+  const bool chain = role == Cf::kChain, loader = role == Cf::kLoader, producer = role == Cf::kProducer;
+  const bool coef = role == Cf::kCoef, zwarp = role == Cf::kRight;
+  const int p = Cf::index(warp) * 32 + lane;  // thread within the role
   const int nx = M.nx, ny = M.ny;
   const int n = DIR == 0 ? nx : ny, nlines = DIR == 0 ? ny : nx, line0 = blockIdx.x * NL;
   const int m = split_point(n);
@@ -230,12 +245,11 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
   };
   LUState<LP> lu;
   lu.reset();
-  // Cell s of this lane's chunk in the band stage B (LUState::step's
-  // operations): its right side here, or (beta, 1/mu) for the right side's
-  // warp.  beta and tc = c - a d'' of the next cell need only values of the
-  // cells before this one: they are formed while this cell's pivot is
-  // inverted, out of the chain.
   constexpr int kF = C * 2 * NL;
+  // Cell s of this lane's chunk in the band stage B (LUState::step's
+  // operations), FP32.  beta and tc = c - a d'' of the next cell need only
+  // values of the cells before this one: they are formed while this cell's
+  // pivot is inverted, out of the chain.
   LP beta = LP(0), tc = LP(0);
   auto eliminate = [&](int s, bool next, const LP* B, LP* Q, LP& chk) {
     const LP* b = B + s * 2 * NL + lane;
@@ -245,29 +259,125 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
       tc = b[2 * NL + 2 * kF] - b[2 * NL] * lu.d1;
     }
     const LP inv = rcp3(mu), g = dg * inv, dl = b[4 * kF] * inv;
-    pivot_check(mu, inv, chk, bad);
+    const LP z = (b[5 * kF] - b[0] * lu.z2 - be * lu.z1) * inv;
+    chk = fma(mu, inv, chk);
     lu.g2 = lu.g1;
     lu.d2 = lu.d1;
+    lu.z2 = lu.z1;
     lu.g1 = g;
     lu.d1 = dl;
+    lu.z1 = z;
     Q[s * NL] = g;
     Q[C * NL + s * NL] = dl;
-    if constexpr (Cf::Z) {
-      S.s.f.bi[s][lane][0] = be;
-      S.s.f.bi[s][lane][1] = inv;
-    } else {
-      const LP z = (b[5 * kF] - b[0] * lu.z2 - be * lu.z1) * inv;
-      lu.z2 = lu.z1;
-      lu.z1 = z;
-      Q[2 * C * NL + s * NL] = z;
+    Q[2 * C * NL + s * NL] = z;
+  };
+  // The same in FP64, a chunk of len cells (0: none of this lane's): the three
+  // warps meet at named barriers of 64 threads, 5 (1/mu and g of a cell: the
+  // chain to the coefficients' warp), 6 (the next cell's coefficients: back) and
+  // 1 .. 4 (a sub-chunk's beta and 1/mu: the chain to the right side).  All their
+  // lanes go through every cell of the chunk, so that the barriers match; cells
+  // at len and beyond are computed from what the band buffer holds and dropped.
+  LP* const ig = S.s.f.ig[lane < 2 * NL ? lane : 0];
+  LP* const co = S.s.f.co[lane < 2 * NL ? lane : 0];
+  const int bl = lane < 2 * NL ? lane : 0;
+  auto chain64 = [&](int len, LP* Q) {
+    asm volatile("bar.sync 6, 64;" ::: "memory");
+    LP be = co[0], t = co[1], dg = co[2], be1 = co[3], t1 = co[4], g = lu.g1;
+#pragma unroll 1
+    for (int s0 = 0; s0 < C; s0 += Cf::SUB) {
+#pragma unroll
+      for (int i = 0; i < Cf::SUB; ++i) {
+        const int s = s0 + i;
+        const LP mu = t - be * g, inv = rcp3(mu);
+        if (s > 0) {
+          asm volatile("bar.sync 6, 64;" ::: "memory");
+          be1 = co[0];
+          t1 = co[1];
+          dg = co[2];
+        }
+        g = dg * inv;
+        if (lane < 2 * NL) {
+          ig[0] = inv;
+          ig[1] = g;
+          S.s.f.bi[s][lane][0] = be;
+          S.s.f.bi[s][lane][1] = inv;
+        }
+        asm volatile("bar.arrive 5, 64;" ::: "memory");
+        if (s < len) {
+          Q[s * NL] = g;
+          lu.g1 = g;
+        }
+        be = be1;
+        t = t1;
+      }
+      asm volatile("bar.arrive %0, 64;" ::"r"(1 + s0 / Cf::SUB) : "memory");
     }
   };
-  auto right_side = [&](int s, const LP* B, LP* Q) {
-    const LP* b = B + s * 2 * NL + lane;
-    const LP z = (b[5 * kF] - b[0] * lu.z2 - S.s.f.bi[s][lane][0] * lu.z1) * S.s.f.bi[s][lane][1];
-    lu.z2 = lu.z1;
-    lu.z1 = z;
-    Q[2 * C * NL + s * NL] = z;
+  auto coef64 = [&](int len, const LP* B, LP* Q) {
+    const LP* b = B + bl;
+    LP be1;
+    {
+      const LP be0 = b[kF] - b[0] * lu.g2, t0 = b[2 * kF] - b[0] * lu.d2;
+      const LP a1 = b[2 * NL], dg0 = b[3 * kF] - be0 * lu.d1;
+      be1 = b[2 * NL + kF] - a1 * lu.g1;
+      const LP t1 = b[2 * NL + 2 * kF] - a1 * lu.d1;
+      if (lane < 2 * NL) {
+        co[0] = be0;
+        co[1] = t0;
+        co[2] = dg0;
+        co[3] = be1;
+        co[4] = t1;
+      }
+    }
+    asm volatile("bar.arrive 6, 64;" ::: "memory");
+#pragma unroll 6
+    for (int s = 0; s < C; ++s) {
+      asm volatile("bar.sync 5, 64;" ::: "memory");
+      const LP inv = ig[0], g = ig[1], dl = b[4 * kF] * inv;
+      LP be2 = LP(0);
+      if (s + 1 < C) {
+        const LP dgn = b[2 * NL + 3 * kF] - be1 * dl;
+        LP t2 = LP(0);
+        if (s + 2 < C) {
+          be2 = b[4 * NL + kF] - b[4 * NL] * g;
+          t2 = b[4 * NL + 2 * kF] - b[4 * NL] * dl;
+        }
+        if (lane < 2 * NL) {
+          co[0] = be2;
+          co[1] = t2;
+          co[2] = dgn;
+        }
+        asm volatile("bar.arrive 6, 64;" ::: "memory");
+      }
+      if (s < len) {
+        Q[C * NL + s * NL] = dl;
+        lu.g2 = lu.g1;
+        lu.d2 = lu.d1;
+        lu.g1 = g;
+        lu.d1 = dl;
+      }
+      be1 = be2;
+      b += 2 * NL;
+    }
+  };
+  auto right64 = [&](int len, const LP* B, LP* Q) {
+#pragma unroll 1
+    for (int s0 = 0; s0 < C; s0 += Cf::SUB) {
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + s0 / Cf::SUB) : "memory");
+#pragma unroll
+      for (int i = 0; i < Cf::SUB; ++i) {
+        const int s = s0 + i;
+        const LP* b = B + s * 2 * NL + bl;
+        const LP inv = S.s.f.bi[s][bl][1];
+        const LP z = (b[5 * kF] - b[0] * lu.z2 - S.s.f.bi[s][bl][0] * lu.z1) * inv;
+        if (s < len) {
+          lu.z2 = lu.z1;
+          lu.z1 = z;
+          Q[2 * C * NL + s * NL] = z;
+          if (zero_or_nonfinite(inv)) bad = 1;
+        }
+      }
+    }
   };
   if (loader) {
     for (int q = 0; q < D - 1; ++q) issue_fwd(q);
@@ -285,51 +395,36 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
       const int len = mine && q < nchh(ch) ? c1_of(ch, q) - c0_of(ch, q) : 0;
       const LP* B = &S.s.f.band[q & 1][0][0][0];
       LP* Q = fac + fac_slab<C>(NL, blockIdx.x, ch & 1, q, nch) + cl;
-      const bool whole = __all_sync(0xffffffffu, len == C || len == 0);
-      if (chain) {
+      if constexpr (Cf::Z) {
+        if (chain)
+          chain64(len, Q);
+        else if (coef)
+          coef64(len, B, Q);
+        else
+          right64(len, B, Q);
+      } else {
         LP chk = LP(0);
         if (len) {
           beta = B[kF + lane] - B[lane] * lu.g2;
           tc = B[2 * kF + lane] - B[lane] * lu.d2;
         }
-#pragma unroll 1
-        for (int s0 = 0; s0 < C; s0 += Cf::Z ? Cf::SUB : C) {
-          constexpr int kN = Cf::Z ? Cf::SUB : C;
-          if (whole) {
-            if (len) {
+        if (__all_sync(0xffffffffu, len == C || len == 0)) {
+          if (len) {
 #pragma unroll
-              for (int i = 0; i < kN; ++i) eliminate(s0 + i, s0 + i + 1 < C, B, Q, chk);
-            }
-          } else {
-#pragma unroll 2
-            for (int i = 0; i < kN; ++i)
-              if (s0 + i < len) eliminate(s0 + i, s0 + i + 1 < len, B, Q, chk);
+            for (int s = 0; s < C; ++s) eliminate(s, s + 1 < C, B, Q, chk);
           }
-          // hand the sub-chunk over (one barrier id each, reused after the tick's barrier)
-          if constexpr (Cf::Z) asm volatile("bar.arrive %0, 64;" ::"r"(1 + s0 / Cf::SUB) : "memory");
+        } else {
+#pragma unroll 2
+          for (int s = 0; s < C; ++s)
+            if (s < len) eliminate(s, s + 1 < len, B, Q, chk);
         }
         if (!(chk == chk)) bad = 1;
-      } else if constexpr (Cf::Z) {  // the right side's warp
-#pragma unroll 1
-        for (int s0 = 0; s0 < C; s0 += Cf::SUB) {
-          asm volatile("bar.sync %0, 64;" ::"r"(1 + s0 / Cf::SUB) : "memory");
-          if (whole) {
-            if (len) {
-#pragma unroll
-              for (int i = 0; i < Cf::SUB; ++i) right_side(s0 + i, B, Q);
-            }
-          } else {
-#pragma unroll 1
-            for (int i = 0; i < Cf::SUB; ++i)
-              if (s0 + i < len) right_side(s0 + i, B, Q);
-          }
-        }
       }
     }
     __syncthreads();
   }
   // ---------------- seam ----------------
-  if (chain && lane < 2 * NL) {
+  if ((Cf::Z ? coef : chain) && lane < 2 * NL) {
     LUState<LP>& o = S.seam[lane];
     o.g1 = lu.g1;
     o.d1 = lu.d1;
