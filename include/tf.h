@@ -367,7 +367,7 @@ int tf_residual_noalloc(const tf_params* p, void* stream, const double* h_k,
  * g_h: device output grid (not aliasing h_old, g or h_new); g_kappa,
  * g_theta: host outputs or NULL (g_theta = g_kappa dkappa/dtheta_c when
  * kappa was derived from the contact angle, else 0).  K: 1..64.
- * Workspace (3K + 19 grids) is allocated on first use and kept by the
+ * Workspace (3K + 16 grids and the solves' factors, about 4 more) is allocated on first use and kept by the
  * context.  Synchronises the context's stream.  Returns TF_OK, TF_ERR_ARG,
  * TF_ERR_NOMEM or TF_ERR_CUDA (or a forward iteration's error).         */
 int tf_adjoint_step(tf_ctx* ctx, const double* h_old, double dt, int K, const double* g,

@@ -37,7 +37,19 @@ struct Ops {
   // The graph of a whole ensemble film run (tf_ensemble_dev.cuh) for
   // contexts on the FP32-bulk power-law twisted path; NULL for the others.
   cudaError_t (*ens_graph)(tf_ctx& c, EnsDev* e, cudaGraphExec_t* out);
+  // Transposed line solves of the adjoint (FP64; NULL for the others): A^T x = r
+  // along the lines of direction dir (0: x), A's diagonals band[d * N + cell];
+  // fac: factor scratch of solve_t_scratch() doubles.
+  cudaError_t (*solve_t)(tf_ctx& c, int dir, const double* band, const double* r, double* out, double* fac, cudaStream_t s);
 };
+
+// Doubles of factor scratch for solve_t in either direction (blocks of up to
+// 16 lines).
+inline size_t solve_t_scratch(int nx, int ny) {
+  const size_t x = fac_slab<kCX>(16, (ny + 15) / 16, 0, 0, chunks_per_half<kCX>(nx));
+  const size_t y = fac_slab<kRY>(16, (nx + 15) / 16, 0, 0, chunks_per_half<kRY>(ny));
+  return x > y ? x : y;
+}
 
 extern const Ops ops_fp64;
 extern const Ops ops_f32b;

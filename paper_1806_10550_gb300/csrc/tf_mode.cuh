@@ -71,6 +71,10 @@ template <class Mode> struct Launch {
     cudaError_t e = allow(k_narrow_sweep<Mode, NL, 0, DEV, GEN>, smem_n<NL, 0>);
     return e ? e : allow(k_narrow_sweep<Mode, NL, 1, DEV, GEN>, smem_n<NL, 1>);
   }
+  template <int NL> static cudaError_t prepare_solve_t() {
+    cudaError_t e = allow(k_narrow_sweep<Mode, NL, 0, false, false, true>, smem_n<NL, 0>);
+    return e ? e : allow(k_narrow_sweep<Mode, NL, 1, false, false, true>, smem_n<NL, 1>);
+  }
   template <bool DEV, bool GEN> static cudaError_t prepare_sweeps() {
     cudaError_t e;
     if constexpr (kWide<GEN>) {
@@ -96,6 +100,9 @@ template <class Mode> struct Launch {
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsExplicit>, A, (int)smem_rhs))) return e;
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsBoth>, A, (int)smem_rhs))) return e;
     if ((e = prepare_sweeps<false, false>()) || (e = prepare_sweeps<false, true>())) return e;
+    if constexpr (!kF32B) {
+      if ((e = prepare_solve_t<4>()) || (e = prepare_solve_t<8>()) || (e = prepare_solve_t<16>())) return e;
+    }
     const cudaFuncAttribute C = cudaFuncAttributePreferredSharedMemoryCarveout;
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsExplicit>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
     if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsBoth>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
@@ -170,6 +177,30 @@ template <class Mode> struct Launch {
     k_rhs<Mode, kRhsBoth><<<grid, 256, smem_rhs, c.stream>>>(c.mk, rhs_consts<HP>(c.mk, step(c, dt), true), u_old,
                                                              (HP*)c.bn, (LP*)c.w, (LP*)c.ulp, c.px);
     return cudaGetLastError();
+  }
+  // A^T x = r along every line of direction dir (FP64): x in `out`, factors in
+  // fac (fac_slab of 16 lines a block at most).
+  template <int NL, int DIR> static cudaError_t solve_t_nl(tf_ctx& c, const GivenBand& gb, double* fac, cudaStream_t s) {
+    const int lines = DIR == 0 ? c.mk.ny : c.mk.nx;
+    k_narrow_sweep<Mode, NL, DIR, false, false, true><<<(lines + NL - 1) / NL, NarrowCfg<LP, NL>::NT, smem_n<NL, DIR>, s>>>(
+        c.mk, LineK<LP>(), nullptr, nullptr, nullptr, (LP*)fac, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+        RunAhead{nullptr, 0}, gb);
+    return cudaGetLastError();
+  }
+  template <int DIR> static cudaError_t solve_t_dir(tf_ctx& c, const GivenBand& gb, double* fac, cudaStream_t s) {
+    switch (DIR == 0 ? c.nlx : c.nly) {
+      case 4: return solve_t_nl<4, DIR>(c, gb, fac, s);
+      case 8: return solve_t_nl<8, DIR>(c, gb, fac, s);
+      default: return solve_t_nl<16, DIR>(c, gb, fac, s);
+    }
+  }
+  static cudaError_t solve_t_c(tf_ctx& c, int dir, const double* band, const double* r, double* out, double* fac, cudaStream_t s) {
+    if constexpr (kF32B) {
+      return cudaErrorNotSupported;
+    } else {
+      const GivenBand gb = {band, r, out, c.N};
+      return dir == 0 ? solve_t_dir<0>(c, gb, fac, s) : solve_t_dir<1>(c, gb, fac, s);
+    }
   }
   // film the sweeps stage: u_k itself in FP64, its FP32 copy (written by
   // k_rhs of the same iteration) in FP32-bulk
@@ -316,6 +347,7 @@ template <class Mode> Ops make_ops() {
   o.ysweep = &L::ysweep_c;
   o.w_to_f64 = &L::w_to_f64_c;
   o.ens_graph = L::kF32B ? &L::ens_graph_c : nullptr;
+  o.solve_t = L::kF32B ? nullptr : &L::solve_t_c;
   return o;
 }
 

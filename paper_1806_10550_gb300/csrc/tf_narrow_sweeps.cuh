@@ -154,17 +154,28 @@ __device__ __forceinline__ void narrow_rows(T* dst, const T* __restrict__ base, 
   for (int r = p / WP; r < nr; r += RG) cpT(dst + r * DP + c, base + (size_t)r * nx + c);
 }
 
+// A line system given by its matrix instead of a film (FP64): A^T x = r with A's
+// diagonals in band[d * N + cell] (the coefficient of line cell t + d - 2 in row
+// t) and x to `out`.
+struct GivenBand {
+  const double* band;
+  const double* r;
+  double* out;
+  size_t N;
+};
+
 // DIR 0: the x sweep (lines are rows; w holds the right sides and receives
 // the solution).  DIR 1: the y sweep (lines are columns; w is the right side,
 // u_{k+1} = u_k + v goes to unew and v to vout when asked for).  DEV and GEN
 // as for k_ysweep.
-template <class Mode, int NL, int DIR, bool DEV, bool GEN>
+// GIVEN: the producers read the band of A^T from gb.
+template <class Mode, int NL, int DIR, bool DEV, bool GEN, bool GIVEN = false>
 __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::kSweepBlocks)
     k_narrow_sweep(ModelK M, LineK<typename Mode::LP> Lp, const double* __restrict__ up,
                    const typename Mode::LP* __restrict__ ul, typename Mode::LP* w, typename Mode::LP* __restrict__ fac,
                    double* __restrict__ unp, double* __restrict__ vout, PartX* __restrict__ partx,
                    PartY* __restrict__ party, const LineK<typename Mode::LP>* __restrict__ Ld,
-                   const double* const* __restrict__ uio, RunAhead ra) {
+                   const double* const* __restrict__ uio, RunAhead ra, GivenBand gb = {}) {
   if (ra.over()) return;
   typedef typename Mode::LP LP;
   typedef NarrowCfg<LP, NL> Cf;
@@ -195,6 +206,7 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
 
   // ---------------- forward ----------------
   auto issue_fwd = [&](int q) {
+    if (GIVEN) return;
     const int slot = q % D;
     for (int h = 0; h < 2; ++h) {
       if (q >= nchh(h)) continue;
@@ -221,6 +233,29 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
     LP* P = &S.s.f.band[t & 1][0][h ? c1 - 1 - ia : ia - c0][h * NL + c];
     const int ks = h ? -2 * NL : 2 * NL;
     constexpr int kF = C * 2 * NL;
+    if constexpr (GIVEN) {  // row t of A^T is column t of A; the loads of all G cells in flight together
+      const size_t step = DIR == 0 ? 1 : (size_t)nx, line = DIR == 0 ? (size_t)(line0 + c) * nx : (size_t)(line0 + c);
+      LP v[G][6];
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        const int t0 = ia + i;
+        if (t0 >= ib) continue;
+#pragma unroll
+        for (int d = 0; d < 5; ++d) {
+          const int row = t0 + d - 2;
+          v[i][d] = row >= 0 && row < n ? __ldg(gb.band + (size_t)(4 - d) * gb.N + line + (size_t)row * step) : LP(0);
+        }
+        v[i][5] = __ldg(gb.r + line + (size_t)t0 * step);
+      }
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        if (ia + i >= ib) continue;
+        LP* q = P + i * ks;
+        for (int d = 0; d < 5; ++d) q[d * kF] = h ? v[i][4 - d] : v[i][d];
+        q[5 * kF] = v[i][5];
+      }
+      return;
+    }
     const LP* T = S.s.f.ut[slot][h] + (DIR == 0 ? (c + 1) * Cf::XP + ia - c0 + 4 : (ia - c0 + 2) * Cf::YP + c + 4);
     const LP* W = S.s.f.rt[slot][h] + (DIR == 0 ? c * Cf::XP + ia - c0 : (ia - c0) * NL + c);
     auto A = [&](int s, int dr, int dc) {
@@ -448,7 +483,7 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
       const int q = nchh(h) - 1 - bq;
       if (bq < nch && q >= 0)
         copy_span<Cf::NLD, LP, 3 * C * NL>(S.s.b.ft[bq % R][h], fac + fac_slab<C>(NL, blockIdx.x, h, q, nch), 3 * C * NL, p);
-      if constexpr (DIR == 1) {
+      if constexpr (DIR == 1 && !GIVEN) {
         const int v = nchh(h) - 1 - bu;
         if (bu >= 0 && bu < nch && v >= 0) {
           const int r0 = c0_of(h, v);
@@ -532,7 +567,9 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
           const int q = nchh(h) - 1 - bq;
           if (q < 0) continue;
           const int c0 = c0_of(h, q), nc = c1_of(h, q) - c0;
-          LP* dst = w + (size_t)line0 * nx + c0;
+          LP* dst;
+          if constexpr (GIVEN) dst = gb.out + (size_t)line0 * nx + c0;
+          else dst = w + (size_t)line0 * nx + c0;
           const LP* X = &S.s.b.xb[bq & 1][h][0][0];
 #pragma unroll
           for (int i = 0; i < (NL * C + NP - 1) / NP; ++i) {
@@ -554,6 +591,10 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
               const int r = rg + RG * i;
               if (r >= nr) break;
               const LP x = S.s.b.xb[bq & 1][h][r][c];
+              if constexpr (GIVEN) {
+                gb.out[(size_t)(r0 + r) * nx + col] = x;
+                continue;
+              }
               const double uk = S.s.b.ukt[bq % R][h][r][c];
               const double un = uk + widen_exact(x);
               const size_t idx = (size_t)(r0 + r) * nx + col;
@@ -569,6 +610,7 @@ __global__ void __launch_bounds__((NarrowCfg<typename Mode::LP, NL>::NT), Mode::
     }
     __syncthreads();
   }
+  if constexpr (GIVEN) return;
   // ---------------- block reduction ----------------
   for (int o = 16; o > 0; o >>= 1) {
     const LP e2 = __shfl_xor_sync(0xffffffffu, err, o);
