@@ -58,7 +58,7 @@ def peaks() -> dict:
 # sources are unchanged (current_counters), so an edited kernel reads null
 # until it is counted again.
 CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_1806_10550_gb300", "csrc")
-_SWEEP_SOURCES = ["tf_line_sweeps.cuh", "tf_sweeps.cuh", "tf_kernels.cuh", "tf_numeric.cuh"]
+_SWEEP_SOURCES = ["tf_narrow_sweeps.cuh", "tf_line_sweeps.cuh", "tf_sweeps.cuh", "tf_kernels.cuh", "tf_numeric.cuh"]
 KERNEL_SOURCES = {
     ("f32b", "rhs"): ["tf_rhs_packed.cuh", "tf_kernels.cuh", "tf_numeric.cuh"],
     ("f32b", "explicit"): ["tf_rhs_packed.cuh", "tf_kernels.cuh", "tf_numeric.cuh"],

@@ -405,6 +405,7 @@ int rev_workspace(tf_ctx* c, int K, bool iterates, RevWork* w) {
       cudaGetLastError();
       return TF_ERR_NOMEM;
     }
+    if (c->ops->solve_t_prepare() != cudaSuccess) return TF_ERR_CUDA;
     c->adj_bytes = bytes;
   }
   double* base = (double*)c->adj_ws;

@@ -537,7 +537,6 @@ void tf_destroy(tf_ctx* c) {
   cudaFree(c->px);
   cudaFree(c->py);
   cudaFree(c->dsc);
-  cudaFree(c->mark);
   for (int k = 0; k < 2; ++k)
     if (c->it_ev[k]) cudaEventDestroy(c->it_ev[k]);
   if (c->hsc) cudaFreeHost(c->hsc);
@@ -614,13 +613,18 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
   mk.pol_A1 = p->pol_A_SiOx;
   mk.pol_A2 = p->pol_A_Si;
   mk.pol_d = p->pol_d;
-  c->grid_rx = (p->nx + 31) / 32;
-  c->grid_ry = (p->ny + 31) / 32;
+  // 32 x 32 tiles spend least on halos; a film of fewer tiles than SMs runs in
+  // tiles of 16 (FP64, us in tiles of 32 and 16: 64^2 19 and 11, 256^2 20 and 14)
+  c->rhs_tile = (long)((p->nx + 31) / 32) * ((p->ny + 31) / 32) < kSMs ? 16 : 32;
+  c->grid_rx = (p->nx + c->rhs_tile - 1) / c->rhs_tile;
+  c->grid_ry = (p->ny + c->rhs_tile - 1) / c->rhs_tile;
   c->packed_rhs = p->precision != TF_FP64 && p->model == TF_MODEL_POWERLAW && p->n == 3 && p->m == 2;
   set_shapes(*c, 0);
   c->grid_st_x = (p->nx + 15) / 16;
   c->grid_st_y = (p->ny + 15) / 16;
-  c->grid_stats = 1216;  // 8 blocks of 256 threads per SM on 152 SMs
+  // 8 blocks of 256 threads per SM, four cells a thread at least: a small film's
+  // statistics are no longer than their reduction
+  c->grid_stats = c->N < (size_t)8 * kSMs * 1024 ? (int)((c->N + 1023) / 1024) : 8 * kSMs;
   {
     int a = c->n_rhs_parts + c->grid_x, b = c->grid_st_x * c->grid_st_y;
     c->n_px = a > b ? a : b;
@@ -633,8 +637,6 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
   const size_t facx = tf::fac_slab<tf::kCX>(32, (p->ny + 31) / 32, 0, 0, tf::chunks_per_half<tf::kCX>(p->nx));
   const size_t facy = tf::fac_slab<tf::kRY>(32, (p->nx + 31) / 32, 0, 0, tf::chunks_per_half<tf::kRY>(p->ny));
   int r = TF_OK;
-  cudaError_t e = c->ops->prepare();
-  if (e != cudaSuccess) r = cuda_fail(e);
   if (!r) r = dalloc(&c->bn, c->N * hp);
   if (!r) r = dalloc(&c->w, c->N * lp);
   if (!r && lp != sizeof(double)) r = dalloc(&c->ulp, c->N * lp);
@@ -646,6 +648,8 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
     }
     c->part = c->packed_rhs && solver == TF_SOLVER_PARTITIONED;
   }
+  cudaError_t e = c->ops->prepare(*c);
+  if (e != cudaSuccess) r = cuda_fail(e);
   c->nsx = tf::part::nseg_x(p->nx);
   c->nsy = tf::part::nseg_y(p->ny);
   if (c->part) {
@@ -664,13 +668,15 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
   if (!r) r = dalloc(&c->ubuf2, c->N * sizeof(double));
   if (!r) r = dalloc(&c->px, (size_t)c->n_px * sizeof(tf::PartX));
   if (!r) r = dalloc(&c->py, (size_t)c->n_py * sizeof(tf::PartY));
-  if (!r) r = dalloc(&c->dsc, sizeof(Scalars));
+  if (!r) r = dalloc(&c->dsc, 2 * sizeof(Scalars));  // the scalars, and the steps' mark
+  if (!r) {
+    c->mark = (unsigned*)(c->dsc + 1);
+    if (cudaMemsetAsync(c->mark, 0, sizeof(unsigned), c->stream) != cudaSuccess) r = TF_ERR_CUDA;
+  }
   if (!r) {
     e = cudaMallocHost((void**)&c->hsc, 3 * sizeof(Scalars));
     if (e != cudaSuccess) r = cuda_fail(e);
   }
-  if (!r) r = dalloc(&c->mark, sizeof(int));
-  if (!r && cudaMemset(c->mark, 0, sizeof(int)) != cudaSuccess) r = TF_ERR_CUDA;
   for (int k = 0; k < 2 && !r; ++k) {
     e = cudaEventCreateWithFlags(&c->it_ev[k], cudaEventDisableTiming);
     if (e != cudaSuccess) r = cuda_fail(e);

@@ -24,7 +24,7 @@ struct EnsDev;
 
 struct Ops {
   size_t hp_bytes, lp_bytes;
-  cudaError_t (*prepare)();
+  cudaError_t (*prepare)(tf_ctx& c);
   cudaError_t (*explicit_part)(tf_ctx& c, const double* u_old, double dt);
   // explicit part plus the first iteration's right side (u_0 = u_old)
   cudaError_t (*explicit_rhs0)(tf_ctx& c, const double* u_old, double dt);
@@ -39,7 +39,9 @@ struct Ops {
   cudaError_t (*ens_graph)(tf_ctx& c, EnsDev* e, cudaGraphExec_t* out);
   // Transposed line solves of the adjoint (FP64; NULL for the others): A^T x = r
   // along the lines of direction dir (0: x), A's diagonals band[d * N + cell];
-  // fac: factor scratch of solve_t_scratch() doubles.
+  // fac: factor scratch of solve_t_scratch() doubles; solve_t_prepare once
+  // before the first.
+  cudaError_t (*solve_t_prepare)();
   cudaError_t (*solve_t)(tf_ctx& c, int dir, const double* band, const double* r, double* out, double* fac, cudaStream_t s);
 };
 
@@ -103,7 +105,7 @@ struct tf_ctx {
   int nlx, nly;    // lines per block of the x and y sweeps
   int grid_x;      // blocks of the x sweep (nlx rows each)
   int grid_y;      // blocks of the y sweep (nly columns each)
-  int grid_rx, grid_ry;      // 2-D residual grid (32 x 32 tiles)
+  int rhs_tile, grid_rx, grid_ry;  // 2-D residual grid (16 x 16 or 32 x 32 tiles)
   int grid_pkx;              // packed FP32-bulk residual: blocks of kRhsStripWarps strip segments
   int strip_n, strip_rows;   // its strips across x and rows per segment
   bool packed_rhs;           // FP32-bulk with the (3, 2) power law: packed residual kernel
@@ -131,8 +133,8 @@ struct tf_ctx {
   tf::Scalars* dsc;
   tf::Scalars* hsc;  // pinned, 3: the last reduction's; two iterations in flight (see step())
   tf::RunAhead ahead;  // of the iteration being queued
-  int* mark;         // RunAhead's mark
-  int step_no;       // number of the step in flight
+  unsigned* mark;    // RunAhead's mark
+  unsigned step_no;  // number of the step in flight
   cudaEvent_t it_ev[2];  // ends of the two iterations in flight
   tf_timing timing;
   cudaEvent_t ev[8];  // 0-4 iteration timing, 5-6 explicit-part timing, 7 work done (ensembles)

@@ -141,6 +141,7 @@ __device__ __forceinline__ double rcp3(double x) {
 __device__ __forceinline__ float rcp3(float x) { return rcp(x); }
 
 TF_HD df64 rcp(df64 x) { return df_rcp(x); }
+__device__ __forceinline__ df64 rcp3(df64 x) { return rcp(x); }
 
 template <class T> TF_HD T one();
 template <> TF_HD double one<double>() { return 1.0; }
@@ -469,7 +470,7 @@ __device__ __forceinline__ void stencil_cells(StencilSmem<HP, TR, TC>& S, const 
     HP d = ((S.u[r + 1][c + 2] - uc) + (S.u[r + 1][c] - uc)) +
            ((S.u[r + 2][c + 1] - uc) + (S.u[r][c + 1] - uc));
     S.lap[r][c] = d * inv_ds2;
-    HP s = rcp(uc);
+    HP s = rcp3(uc);
     HP f0, f1;
     mobility(mc, uc, s, f0, f1);
     S.s[r][c] = s;
@@ -702,8 +703,8 @@ static __global__ void __launch_bounds__(256)
 // at once.  *mark == step says that step number `step` has ended; mark NULL
 // where nothing runs ahead.
 struct RunAhead {
-  const int* mark;
-  int step;
+  const unsigned* mark;
+  unsigned step;
   __device__ __forceinline__ bool over() const { return mark && *mark == step; }
 };
 
@@ -719,7 +720,7 @@ TF_HD int classify_iteration(const Scalars& s, int it, int fixed_iter, double to
 // mark when it is the last.
 static __global__ void __launch_bounds__(256)
     k_iteration_end(const PartX* __restrict__ px, int nx_part, const PartY* __restrict__ py, int ny_part,
-                    Scalars* __restrict__ out, RunAhead ra, int* mark, int it, int fixed_iter, double tol) {
+                    Scalars* __restrict__ out, RunAhead ra, unsigned* mark, int it, int fixed_iter, double tol) {
   if (ra.over()) return;
   Scalars s;
   if (!finalize_block(px, nx_part, py, ny_part, s)) return;

@@ -17,7 +17,20 @@ template <class Mode> struct Launch {
   typedef typename Mode::HP HP;
   typedef typename Mode::LP LP;
   static constexpr size_t smem_stencil = sizeof(StencilSmem<HP, 16, 16>);
-  static constexpr size_t smem_rhs = sizeof(RhsSmem<HP, 32>);
+  template <int T> static constexpr size_t smem_rhs = sizeof(RhsSmem<HP, T>);
+  // k_rhs in the context's tiles
+  template <int KIND> static cudaError_t launch_rhs(tf_ctx& c, const RhsK<HP>& K, const double* u, RunAhead ra) {
+    const dim3 grid(c.grid_rx, c.grid_ry);
+    if (c.rhs_tile == 16)
+      k_rhs<Mode, KIND, 16><<<grid, 256, smem_rhs<16>, c.stream>>>(c.mk, K, u, (HP*)c.bn, (LP*)c.w, (LP*)c.ulp, c.px, ra);
+    else
+      k_rhs<Mode, KIND, 32><<<grid, 256, smem_rhs<32>, c.stream>>>(c.mk, K, u, (HP*)c.bn, (LP*)c.w, (LP*)c.ulp, c.px, ra);
+    return cudaGetLastError();
+  }
+  template <int KIND> static cudaError_t prepare_rhs() {
+    cudaError_t e = allow(k_rhs<Mode, KIND, 16>, smem_rhs<16>);
+    return e ? e : allow(k_rhs<Mode, KIND, 32>, smem_rhs<32>);
+  }
   static constexpr bool kF32B = std::is_same<Mode, ModeF32B>::value;
   // The kernel, threads and shared memory of a sweep (DIR 0: x, 1: y) in
   // blocks of nl lines, and its launch.  DEV, GEN: see k_ysweep.
@@ -91,25 +104,18 @@ template <class Mode> struct Launch {
     return k;
   }
 
-  static cudaError_t prepare() {
+  // The attributes of the kernels that a context runs (an attribute call a
+  // kernel takes about a microsecond; the ensemble graphs' and the transposed
+  // solves' are set on their first use).
+  static cudaError_t prepare(tf_ctx& c) {
     cudaError_t e;
-    const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if ((e = cudaFuncSetAttribute(k_stencil<Mode, 0>, A, (int)smem_stencil))) return e;
-    if ((e = cudaFuncSetAttribute(k_stencil<Mode, 1>, A, (int)smem_stencil))) return e;
-    if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsResidual>, A, (int)smem_rhs))) return e;
-    if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsExplicit>, A, (int)smem_rhs))) return e;
-    if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsBoth>, A, (int)smem_rhs))) return e;
-    if ((e = prepare_sweeps<false, false>()) || (e = prepare_sweeps<false, true>())) return e;
-    if constexpr (!kF32B) {
-      if ((e = prepare_solve_t<4>()) || (e = prepare_solve_t<8>()) || (e = prepare_solve_t<16>())) return e;
-    }
-    const cudaFuncAttribute C = cudaFuncAttributePreferredSharedMemoryCarveout;
-    if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsExplicit>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
-    if ((e = cudaFuncSetAttribute(k_rhs<Mode, kRhsBoth>, C, (int)cudaSharedmemCarveoutMaxShared))) return e;
+    if (!c.packed_rhs &&
+        ((e = prepare_rhs<kRhsResidual>()) || (e = prepare_rhs<kRhsExplicit>()) || (e = prepare_rhs<kRhsBoth>())))
+      return e;
     if constexpr (kF32B) {
-      if ((e = part::prepare()) || (e = prepare_sweeps<true, false>())) return e;
+      if (c.part) return part::prepare();
     }
-    return cudaFuncSetAttribute(k_rhs<Mode, kRhsResidual>, C, (int)cudaSharedmemCarveoutMaxShared);
+    return power32(c) ? prepare_sweeps<false, false>() : prepare_sweeps<false, true>();
   }
 
   static cudaError_t explicit_part_c(tf_ctx& c, const double* u_old, double dt) {
@@ -121,10 +127,7 @@ template <class Mode> struct Launch {
         return cudaGetLastError();
       }
     }
-    dim3 grid(c.grid_rx, c.grid_ry);
-    k_rhs<Mode, kRhsExplicit><<<grid, 256, smem_rhs, c.stream>>>(c.mk, rhs_consts<HP>(c.mk, step(c, dt), true), u_old,
-                                                         (HP*)c.bn, nullptr, nullptr, nullptr);
-    return cudaGetLastError();
+    return launch_rhs<kRhsExplicit>(c, rhs_consts<HP>(c.mk, step(c, dt), true), u_old, RunAhead{nullptr, 0});
   }
   // G of tf_residual, the partial results of its norm and the film's mass and
   // least height: *npx of them in c.px, *npy in c.py
@@ -155,11 +158,7 @@ template <class Mode> struct Launch {
         return cudaGetLastError();
       }
     }
-    dim3 grid(c.grid_rx, c.grid_ry);
-    k_rhs<Mode, kRhsResidual><<<grid, 256, smem_rhs, c.stream>>>(c.mk, rhs_consts<HP>(c.mk, step(c, dt)), u_k,
-                                                   (HP*)c.bn, (LP*)c.w,
-                                                   (LP*)c.ulp, c.px, c.ahead);
-    return cudaGetLastError();
+    return launch_rhs<kRhsResidual>(c, rhs_consts<HP>(c.mk, step(c, dt)), u_k, c.ahead);
   }
   // b^n of a step and the right side of its first iteration (u_0 = u^n)
   // from one D(u^n); results equal explicit_part_c then rhs_c.
@@ -172,11 +171,7 @@ template <class Mode> struct Launch {
         return cudaGetLastError();
       }
     }
-    c.expl_kernels = 1;
-    dim3 grid(c.grid_rx, c.grid_ry);
-    k_rhs<Mode, kRhsBoth><<<grid, 256, smem_rhs, c.stream>>>(c.mk, rhs_consts<HP>(c.mk, step(c, dt), true), u_old,
-                                                             (HP*)c.bn, (LP*)c.w, (LP*)c.ulp, c.px);
-    return cudaGetLastError();
+    return launch_rhs<kRhsBoth>(c, rhs_consts<HP>(c.mk, step(c, dt), true), u_old, RunAhead{nullptr, 0});
   }
   // A^T x = r along every line of direction dir (FP64): x in `out`, factors in
   // fac (fac_slab of 16 lines a block at most).
@@ -192,6 +187,15 @@ template <class Mode> struct Launch {
       case 4: return solve_t_nl<4, DIR>(c, gb, fac, s);
       case 8: return solve_t_nl<8, DIR>(c, gb, fac, s);
       default: return solve_t_nl<16, DIR>(c, gb, fac, s);
+    }
+  }
+  static cudaError_t solve_t_prepare() {
+    if constexpr (kF32B) {
+      return cudaErrorNotSupported;
+    } else {
+      cudaError_t e;
+      if ((e = prepare_solve_t<4>()) || (e = prepare_solve_t<8>())) return e;
+      return prepare_solve_t<16>();
     }
   }
   static cudaError_t solve_t_c(tf_ctx& c, int dir, const double* band, const double* r, double* out, double* fac, cudaStream_t s) {
@@ -246,7 +250,9 @@ template <class Mode> struct Launch {
       if (!c.packed_rhs || c.part) return cudaErrorNotSupported;
       cudaStream_t s = nullptr;
       cudaGraph_t g = nullptr, B = nullptr, I = nullptr;
-      cudaError_t err = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+      cudaError_t err = prepare_sweeps<true, false>();
+      if (err) return err;
+      err = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
       if (err) return err;
       const cudaStreamCaptureMode md = cudaStreamCaptureModeRelaxed;
       const StripK rk0 = strip_consts(c.mk, step(c, 1.0), false);  // placeholders: read from e
@@ -313,7 +319,7 @@ template <class Mode> struct Launch {
       if ((err = cudaStreamEndCapture(s, &I))) return fail(err);
       // end of the attempt: the result into nxt, its statistics, the controller
       if ((err = cudaStreamBeginCaptureToGraph(s, B, &ni, nullptr, 1, md))) return fail(err);
-      k_ens_copy<<<1024, 256, 0, s>>>(e, c.N);
+      k_ens_copy<<<c.grid_stats < 1024 ? c.grid_stats : 1024, 256, 0, s>>>(e, c.N);
       k_grid_stats<<<c.grid_stats, 256, 0, s>>>(nullptr, c.N, c.py, &e->p.nxt);
       k_ens_step<<<1, 256, 0, s>>>(c.py, c.grid_stats, e, ho);
       if ((err = cudaStreamEndCapture(s, &B))) return fail(err);
@@ -347,6 +353,7 @@ template <class Mode> Ops make_ops() {
   o.ysweep = &L::ysweep_c;
   o.w_to_f64 = &L::w_to_f64_c;
   o.ens_graph = L::kF32B ? &L::ens_graph_c : nullptr;
+  o.solve_t_prepare = L::kF32B ? nullptr : &L::solve_t_prepare;
   o.solve_t = L::kF32B ? nullptr : &L::solve_t_c;
   return o;
 }

@@ -59,7 +59,9 @@ template <class HP, int T> struct RhsSmem {
 // kRhsBoth: both from one D(u^n) -- b^n, and the residual of the step's
 // first iteration (u_0 = u^n) from the stored b^n, as kRhsResidual would
 // form it (gscale the explicit part's, gscale2 the residual's).
-template <class Mode, int KIND>
+// T: the tile, 32 x 32, or 16 x 16 for films that it leaves SMs idle on (a
+// block's tile is a chain of FP64-bound stages; see set_shapes in tf_api.cu).
+template <class Mode, int KIND, int T>
 __global__ void __launch_bounds__(256, 4)  // shared memory allows 4 blocks per SM: up to 64 registers
     k_rhs(ModelK M, RhsK<typename Mode::HP> RK, const double* __restrict__ u,
           typename Mode::HP* __restrict__ bn,
@@ -68,7 +70,7 @@ __global__ void __launch_bounds__(256, 4)  // shared memory allows 4 blocks per 
   if (ra.over()) return;
   typedef typename Mode::HP HP;
   typedef typename Mode::LP LP;
-  constexpr int T = 32, NT = 256;
+  constexpr int NT = 256;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RhsSmem<HP, T>& S = *reinterpret_cast<RhsSmem<HP, T>*>(smem_raw);
   const int tid = threadIdx.x;
@@ -89,7 +91,7 @@ __global__ void __launch_bounds__(256, 4)  // shared memory allows 4 blocks per 
     // the cell itself (reflected tile) and cancels one of the four.
     HP nb = hp_add(hp_add(S.u[r + 1][c + 2], S.u[r + 1][c]), hp_add(S.u[r + 2][c + 1], S.u[r][c + 1]));
     S.lap[r][c] = hp_norm(hp_mul(hp_sub(nb, hp_mul(four, uc)), inv_ds2));
-    HP s = rcp(uc), f0, f1;
+    HP s = rcp3(uc), f0, f1;
     mobility(mc, uc, s, f0, f1);
     S.f0[r][c] = hp_norm(f0);
     S.f1[r][c] = hp_norm(f1);
