@@ -27,9 +27,8 @@ template <class Mode> struct Launch {
       k_rhs<Mode, KIND, 32><<<grid, 256, smem_rhs<32>, c.stream>>>(c.mk, K, u, (HP*)c.bn, (LP*)c.w, (LP*)c.ulp, c.px, ra);
     return cudaGetLastError();
   }
-  template <int KIND> static cudaError_t prepare_rhs() {
-    cudaError_t e = allow(k_rhs<Mode, KIND, 16>, smem_rhs<16>);
-    return e ? e : allow(k_rhs<Mode, KIND, 32>, smem_rhs<32>);
+  template <int KIND> static cudaError_t prepare_rhs(const tf_ctx& c) {
+    return c.rhs_tile == 16 ? allow(k_rhs<Mode, KIND, 16>, smem_rhs<16>) : allow(k_rhs<Mode, KIND, 32>, smem_rhs<32>);
   }
   static constexpr bool kF32B = std::is_same<Mode, ModeF32B>::value;
   // The kernel, threads and shared memory of a sweep (DIR 0: x, 1: y) in
@@ -84,6 +83,9 @@ template <class Mode> struct Launch {
     cudaError_t e = allow(k_narrow_sweep<Mode, NL, 0, DEV, GEN>, smem_n<NL, 0>);
     return e ? e : allow(k_narrow_sweep<Mode, NL, 1, DEV, GEN>, smem_n<NL, 1>);
   }
+  template <bool DEV, bool GEN> static cudaError_t prepare_narrow_nl(int nl) {
+    return nl == 4 ? prepare_narrow<4, DEV, GEN>() : (nl == 8 ? prepare_narrow<8, DEV, GEN>() : prepare_narrow<16, DEV, GEN>());
+  }
   template <int NL> static cudaError_t prepare_solve_t() {
     cudaError_t e = allow(k_narrow_sweep<Mode, NL, 0, false, false, true>, smem_n<NL, 0>);
     return e ? e : allow(k_narrow_sweep<Mode, NL, 1, false, false, true>, smem_n<NL, 1>);
@@ -110,10 +112,14 @@ template <class Mode> struct Launch {
   static cudaError_t prepare(tf_ctx& c) {
     cudaError_t e;
     if (!c.packed_rhs &&
-        ((e = prepare_rhs<kRhsResidual>()) || (e = prepare_rhs<kRhsExplicit>()) || (e = prepare_rhs<kRhsBoth>())))
+        ((e = prepare_rhs<kRhsResidual>(c)) || (e = prepare_rhs<kRhsExplicit>(c)) || (e = prepare_rhs<kRhsBoth>(c))))
       return e;
     if constexpr (kF32B) {
       if (c.part) return part::prepare();
+      if (!power32(c)) {  // one shape whatever runs beside the film (set_shapes)
+        e = prepare_narrow_nl<false, true>(c.nlx);
+        return e || c.nly == c.nlx ? e : prepare_narrow_nl<false, true>(c.nly);
+      }
     }
     return power32(c) ? prepare_sweeps<false, false>() : prepare_sweeps<false, true>();
   }
