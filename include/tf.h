@@ -184,7 +184,11 @@ double tf_kappa(const tf_ctx* ctx);
  *   G   = h_k + theta dt D(h_k) - b^n,
  * with D the discrete flux divergence of eq. GovEqnCell2.
  * h_k, h_old: device grids (may alias).  G: device grid or NULL.
- * out: host struct or NULL (gnorm = max|G|, mass and hmin of h_k).       */
+ * out: host struct or NULL (gnorm = max|G|, NaN left out; mass and hmin of
+ * h_k, hmin over its positive finite heights).  h_k may hold any values, also
+ * ones outside the model's domain (zero, negative, not finite): G is theirs.
+ * In TF_FP32_BULK with the (3, 2) power law the heights of h_old are positive,
+ * 2^-74 <= h_old < 2^63.                                                 */
 int tf_residual(tf_ctx* ctx, const double* h_k, const double* h_old, double dt,
                 double* G, tf_norms* out);
 

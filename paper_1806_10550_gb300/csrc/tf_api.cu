@@ -696,10 +696,13 @@ int tf_init(const tf_params* p, void* stream, tf_ctx** out) {
 int tf_residual(tf_ctx* c, const double* h_k, const double* h_old, double dt, double* G,
                 tf_norms* out) {
   if (!c || !h_k || !h_old || !isfinite(dt)) return TF_ERR_ARG;
-  TF_CK(c->ops->explicit_part(*c, h_old, dt));
-  int npx = 0, npy = 0;
-  TF_CK(c->ops->residual_g(*c, h_k, dt, G ? G : c->ubuf, &npx, &npy));
-  int r = finalize(*c, npx, npy);
+  tf::ReportParts parts;
+  TF_CK(c->ops->report(*c, h_old, h_k, dt, G ? G : c->ubuf, false, &parts));
+  int r = finalize(*c, parts.npx, parts.npy);
+  if (!r && parts.strips && c->hsc->nonfinite) {  // a height that the strips do not take
+    TF_CK(c->ops->report(*c, nullptr, h_k, dt, G ? G : c->ubuf, true, &parts));
+    r = finalize(*c, parts.npx, parts.npy);
+  }
   if (r) return r;
   if (out) {
     out->gnorm = c->hsc->gnorm;

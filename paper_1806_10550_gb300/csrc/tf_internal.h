@@ -22,14 +22,23 @@ namespace tf {
 
 struct EnsDev;
 
+// The partial results that report leaves in px and py, and whether they are
+// the strip kernel's (whose nonfinite flag asks for the tile kernel).
+struct ReportParts {
+  int npx, npy;
+  bool strips;
+};
+
 struct Ops {
   size_t hp_bytes, lp_bytes;
   cudaError_t (*prepare)(tf_ctx& c);
   cudaError_t (*explicit_part)(tf_ctx& c, const double* u_old, double dt);
   // explicit part plus the first iteration's right side (u_0 = u_old)
   cudaError_t (*explicit_rhs0)(tf_ctx& c, const double* u_old, double dt);
-  // G to tf_residual's callers; the numbers of partial results in px and py
-  cudaError_t (*residual_g)(tf_ctx& c, const double* u_k, double dt, double* G, int* npx, int* npy);
+  // tf_residual: b^n of u_old (NULL: it is there), G, its norm and the film's
+  // statistics; tiles: G on the tile kernel, which takes heights of any value
+  cudaError_t (*report)(tf_ctx& c, const double* u_old, const double* u_k, double dt, double* G, bool tiles,
+                        ReportParts* parts);
   cudaError_t (*rhs)(tf_ctx& c, const double* u_k, double dt);
   cudaError_t (*xsweep)(tf_ctx& c, double dt, const double* u_k);
   cudaError_t (*ysweep)(tf_ctx& c, const double* u_k, double dt, double* u_next, double* v_out);

@@ -135,22 +135,38 @@ template <class Mode> struct Launch {
     }
     return launch_rhs<kRhsExplicit>(c, rhs_consts<HP>(c.mk, step(c, dt), true), u_old, RunAhead{nullptr, 0});
   }
-  // G of tf_residual, the partial results of its norm and the film's mass and
-  // least height: *npx of them in c.px, *npy in c.py
-  static cudaError_t residual_c(tf_ctx& c, const double* u_k, double dt, double* G, int* npx, int* npy) {
+  // tf_residual: b^n, G, the partial results of its norm (c.px) and the film's
+  // mass and least height (c.py).  On the strips unless the heights that they
+  // take leave out the precursor's b, below which no film is: such a film would
+  // run on both kernels.
+  static cudaError_t report_c(tf_ctx& c, const double* u_old, const double* u_k, double dt, double* G, bool tiles,
+                              ReportParts* parts) {
+    const dim3 grid(c.grid_st_x, c.grid_st_y), block(16, 16);
     if constexpr (kF32B) {
-      if (c.packed_rhs) {
-        *npx = *npy = c.grid_pkx;
-        k_rhs_strip<kRhsReport><<<c.grid_pkx, kST, 0, c.stream>>>(
-            c.mk, strip_consts(c.mk, step(c, dt), false), u_k, (HP*)c.bn, nullptr, nullptr, c.px, c.strip_n, c.strip_rows,
-            nullptr, nullptr, G, c.py);
-        return cudaGetLastError();
+      if (c.packed_rhs && u_old && !strip_range(c.mk, step(c, dt).expl_dt).has(c.p.b)) {
+        k_stencil<Mode, 0><<<grid, block, smem_stencil, c.stream>>>(c.mk, rhs_consts<HP>(c.mk, step(c, dt), true), u_old,
+                                                                    (HP*)c.bn, nullptr, nullptr);
+        u_old = nullptr;
       }
     }
-    *npx = c.grid_st_x * c.grid_st_y;
-    *npy = c.grid_stats;
+    if (u_old) {
+      const cudaError_t e = explicit_part_c(c, u_old, dt);
+      if (e) return e;
+    }
+    if constexpr (kF32B) {
+      if (c.packed_rhs && !tiles) {
+        const StripRange range = strip_range(c.mk, step(c, dt).theta_dt);
+        if (range.has(c.p.b)) {
+          *parts = ReportParts{c.grid_pkx, c.grid_pkx, true};
+          k_rhs_strip<kRhsReport><<<c.grid_pkx, kST, 0, c.stream>>>(
+              c.mk, strip_consts(c.mk, step(c, dt), false), u_k, (HP*)c.bn, nullptr, nullptr, c.px, c.strip_n, c.strip_rows,
+              nullptr, nullptr, G, c.py, RunAhead{nullptr, 0}, range);
+          return cudaGetLastError();
+        }
+      }
+    }
+    *parts = ReportParts{c.grid_st_x * c.grid_st_y, c.grid_stats, false};
     k_grid_stats<<<c.grid_stats, 256, 0, c.stream>>>(u_k, c.N, c.py);
-    dim3 grid(c.grid_st_x, c.grid_st_y), block(16, 16);
     k_stencil<Mode, 1><<<grid, block, smem_stencil, c.stream>>>(c.mk, rhs_consts<HP>(c.mk, step(c, dt)), u_k, (HP*)c.bn,
                                                                 G, c.px);
     return cudaGetLastError();
@@ -353,7 +369,7 @@ template <class Mode> Ops make_ops() {
   o.prepare = &L::prepare;
   o.explicit_part = &L::explicit_part_c;
   o.explicit_rhs0 = &L::explicit_rhs0_c;
-  o.residual_g = &L::residual_c;
+  o.report = &L::report_c;
   o.rhs = &L::rhs_c;
   o.xsweep = &L::xsweep_c;
   o.ysweep = &L::ysweep_c;

@@ -173,6 +173,37 @@ TF_HD StripK strip_consts(const ModelK& M, const StepK& K, bool expl) {
   return k;
 }
 
+// The heights whose residual the strip arithmetic forms to its 2^-48 of the
+// height, for a step's constants: those whose upper word is one of the `span`
+// from lo on.  Outside them the conversion to float pairs (positive normal
+// values, trailing part included) or a product leaves the floats.  Because the Laplacian is unscaled, that depends on ds: films in
+// metres (h ~ ds ~ 1e-8) have fluxes near 1e-35 here, which the tile kernel
+// carries as fluxes / ds^2.  A flux errs by up to 2^-146 (rounding in the
+// subnormals), or 2^-144 h^2 for h > 1 (f0 times a difference), and a constant
+// below 2^-102 by 2^-126; times gs they have to stay under 2^-50 h.
+struct StripRange {
+  unsigned lo, span;
+  __host__ __device__ bool has(double h) const {  // upper words of negative heights and NaN come last
+    return (unsigned)(bits_of(h) >> 32) - lo < span;
+  }
+};
+inline StripRange strip_range(const ModelK& M, double dt) {  // theta dt or (1 - theta) dt
+  const double ds2 = 1.0 / M.inv_ds2, gs = fabs(0.5 * M.inv_ds2 * M.inv_ds2 * dt);
+  const double A1s = M.A1 * ds2, B1s = M.B1 * ds2;
+  double lo = fmax(0x1p-74, fmax(gs * 0x1p-96, B1s * 0x1p-122));
+  double hi = fmin(0x1p63, fmin(pow(0x1p120 / M.C, 0.25), 0x1p122 / A1s));
+  if (gs > 0.0) hi = fmin(hi, 0x1p94 / gs);
+  if (B1s < 0x1p-102) lo = fmax(lo, gs * 0x1p-75);
+  if (A1s < 0x1p-102 && gs > 0x1p75) hi = 0.0;
+  if (gs > 0.0 && gs < 0x1p-102) {  // gs itself is rounded to 2^-126
+    hi = A1s > 0x1p69 ? 0.0 : fmin(hi, cbrt(0x1p69 / M.C));
+    lo = fmax(lo, B1s * 0x1p-68);
+  }
+  if (!(gs >= 0.0 && lo < hi)) return StripRange{0u, 0u};  // NaN and infinite constants too
+  const unsigned l = (unsigned)(bits_of(lo) >> 32) + 1, h = (unsigned)(bits_of(hi) >> 32);
+  return StripRange{l, h > l ? h - l : 0u};
+}
+
 constexpr int kSW = 60;  // output columns of a strip
 constexpr int kST = 128;  // threads per block
 constexpr int kSWarps = kST / 32;
@@ -376,6 +407,8 @@ __device__ __forceinline__ void strip_copy_bn(float4* dst, const df64* __restric
 // kRhsReport: G of kRhsResidual in FP64 to Gout, its norm in double, and mass
 // and least height of u_k to party (the heights pass through anyway): at 2048^2
 // it takes the place of a 16 x 16-tile kernel of 242 us and a pass of 14 us.
+// party's nonfinite flag says that a height lies outside `range`, where nothing
+// of this is the film's: the caller then runs the tile kernel.
 // Warp w of the grid takes strip w % nstrip and rows [seg_rows * (w /
 // nstrip), + seg_rows); one partial result (max|G|) per block.
 // DEV (the ensemble graphs): the step's constants *RKd and the grid *ud come
@@ -385,7 +418,8 @@ __global__ void __launch_bounds__(kST, 5)
     k_rhs_strip(ModelK M, StripK RKp, const double* __restrict__ up, df64* __restrict__ bn,
                 float* __restrict__ rhs, float* __restrict__ ulp, PartX* __restrict__ part, int nstrip,
                 int seg_rows, const StripK* __restrict__ RKd = nullptr, const double* const* __restrict__ ud = nullptr,
-                double* __restrict__ Gout = nullptr, PartY* __restrict__ party = nullptr, RunAhead ra = {nullptr, 0}) {
+                double* __restrict__ Gout = nullptr, PartY* __restrict__ party = nullptr, RunAhead ra = {nullptr, 0},
+                StripRange range = {0u, 0u}) {
   if (ra.over()) return;
   constexpr bool kB = KIND == kRhsResidual || KIND == kRhsReport;  // reads b^n
   const StripK& RK = DEV ? *RKd : RKp;
@@ -410,7 +444,7 @@ __global__ void __launch_bounds__(kST, 5)
     auto stats = [&](double2 v) {  // the lane's pair of an output row
       auto take = [&](double x) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-        if (!positive_finite_bits(x)) nf = 1;
+        if (!range.has(x)) nf = 1;
         else if (b < hmin) hmin = b;
         mass_add(mass, (unsigned long long)fixed36_of_f64(x));
       };

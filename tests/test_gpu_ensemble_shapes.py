@@ -1,0 +1,83 @@
+"""Ensembles of changing size on the same contexts.
+
+The block shapes of a film's kernels depend on how many lines advance at once.
+A context keeps the graph of each shape it ran in: a film that goes back and
+forth between two sets pays for a graph once per shape, and its results do not
+depend on the set.
+"""
+import time
+
+import pytest
+
+import paper_1806_10550_gb300 as tf
+from paper_1806_10550_gb300 import synthetic as S
+
+pytestmark = pytest.mark.gpu
+
+KAPPA = 1.2061475842818314
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch as T
+    if not T.cuda.is_available():
+        pytest.skip("no CUDA device")
+    tf.library()
+    return T
+
+
+def context(torch, nx, ny):
+    return tf.Context(tf.tf_params_default(nx=nx, ny=ny, ds=3.9, kappa=KAPPA, precision=tf.TF_FP32_BULK),
+                      stream=torch.cuda.Stream())
+
+
+def test_alternating_sets_keep_their_graphs(torch):
+    """One film alone, then among 30 (6000 lines): the call of the film alone
+    right after the other set's takes less than half a graph's build more than
+    the same call repeated (least of 12 each; the build: the least first call
+    of a fresh context, less the repeated call)."""
+    films = [torch.from_numpy(S.spinodal_film(200, 170, 1.0, 0.01, seed=k)).cuda() for k in range(30)]
+    ctxs = [context(torch, 200, 170) for _ in films]
+    torch.cuda.synchronize()
+
+    def alone(ctx):
+        t = time.perf_counter()
+        tf.tf_ensemble_advance([ctx], films[:1], 0.0, 1e30, 1e-3, 1)
+        return time.perf_counter() - t
+
+    first = []
+    for _ in range(4):
+        c = context(torch, 200, 170)
+        first.append(alone(c))
+        c.close()
+    alone(ctxs[0])
+    repeated = min(alone(ctxs[0]) for _ in range(12))
+    build = min(first[1:]) - repeated
+    assert build > 0.0
+    after = []
+    for _ in range(13):
+        tf.tf_ensemble_advance(ctxs, films, 0.0, 1e30, 1e-3, 1)
+        after.append(alone(ctxs[0]))
+    assert min(after[1:]) < repeated + 0.5 * build, (min(after[1:]), repeated, build)
+    for c in ctxs:
+        c.close()
+
+
+def test_results_do_not_depend_on_the_set(torch):
+    """A film advanced in sets of 1, 8, 64, 30 and 1 films against tf_advance
+    over the same attempts."""
+    start = [torch.from_numpy(S.spinodal_film(200, 170, 1.0, 0.01, seed=90 + k)).cuda() for k in range(64)]
+    ctxs = [context(torch, 200, 170) for _ in start]
+    grids = [h.clone() for h in start]
+    ref = start[0].clone()
+    torch.cuda.synchronize()
+    single = tf.Context(tf.tf_params_default(nx=200, ny=170, ds=3.9, kappa=KAPPA, precision=tf.TF_FP32_BULK))
+    a = b = dict(t=0.0, dt=1e-2, streak=0)
+    for n in (1, 8, 64, 30, 1):
+        infos = tf.tf_ensemble_advance(ctxs[:n], grids[:n], a["t"], 1e30, a["dt"], 2, streak=a["streak"])
+        a = infos[0]
+        b, _ = tf.tf_advance(single, ref, b["t"], 1e30, b["dt"], 2, streak=b["streak"])
+        assert a == b
+        assert torch.equal(grids[0], ref)
+    for c in ctxs + [single]:
+        c.close()
