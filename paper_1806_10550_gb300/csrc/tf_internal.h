@@ -29,6 +29,15 @@ struct ReportParts {
   bool strips;
 };
 
+// A film's run as an instantiated graph, and the lines per sweep block and rows
+// per strip segment it was built with.  A context takes one of four shapes by
+// the lines that advance at once (shared_lines in tf_api.cu).
+constexpr int kEnsGraphs = 4;
+struct EnsGraph {
+  cudaGraphExec_t exec;
+  int nlx, nly, rows;
+};
+
 struct Ops {
   size_t hp_bytes, lp_bytes;
   cudaError_t (*prepare)(tf_ctx& c);
@@ -154,6 +163,5 @@ struct tf_ctx {
   // graph engine of tf_ensemble_advance (built on first use)
   tf::EnsDev* ens_dev;        // the film's device-resident controller state
   tf::EnsDev* ens_host;       // pinned staging copy of it
-  cudaGraphExec_t ens_exec;   // the instantiated graph of a whole run
-  int ens_nlx, ens_nly, ens_rows;  // the lines per sweep block and rows per strip segment it was built with
+  tf::EnsGraph ens_graphs[tf::kEnsGraphs];  // the graphs of a whole run, one per block shape it was run in
 };
