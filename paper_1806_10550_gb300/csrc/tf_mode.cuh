@@ -35,43 +35,54 @@ template <class Mode> struct Launch {
   // blocks of nl lines, and its launch.  DEV, GEN: see k_ysweep.
   template <int NL, int DIR> static constexpr size_t smem_n = sizeof(NarrowSmem<LP, NL, DIR>);
   static constexpr size_t smem_x = sizeof(XSmem<LP>), smem_y = sizeof(YSmem<LP>);
-  // whether any film runs in blocks of 32 lines (see sweep_lines and set_lines)
+  // whether any film runs in blocks of 32 lines (see sweep_lines and set_shapes in
+  // tf_api.cu); a context in a block shape without a kernel is refused
   template <bool GEN> static constexpr bool kWide = !(kF32B && GEN);
   template <int NL, bool DEV, bool GEN>
-  static void narrow_x(tf_ctx& c, const LineK<LP>& L, const LP* ul, const LineK<LP>* Ld, cudaStream_t s) {
+  static cudaError_t narrow_x(tf_ctx& c, const LineK<LP>& L, const LP* ul, const LineK<LP>* Ld, cudaStream_t s) {
     k_narrow_sweep<Mode, NL, 0, DEV, GEN><<<c.grid_x, NarrowCfg<LP, NL>::NT, smem_n<NL, 0>, s>>>(
         c.mk, L, nullptr, ul, (LP*)c.w, (LP*)c.fac_x, nullptr, nullptr, c.px + c.n_rhs_parts, nullptr, Ld, nullptr, c.ahead);
+    return cudaGetLastError();
   }
   template <int NL, bool DEV, bool GEN>
-  static void narrow_y(tf_ctx& c, const LineK<LP>& L, const double* u, const LP* ul, double* un, double* v,
+  static cudaError_t narrow_y(tf_ctx& c, const LineK<LP>& L, const double* u, const LP* ul, double* un, double* v,
                        const LineK<LP>* Ld, const double* const* uio, cudaStream_t s) {
     k_narrow_sweep<Mode, NL, 1, DEV, GEN><<<c.grid_y, NarrowCfg<LP, NL>::NT, smem_n<NL, 1>, s>>>(
         c.mk, L, u, ul, (LP*)c.w, (LP*)c.fac_y, un, v, nullptr, c.py, Ld, uio, c.ahead);
+    return cudaGetLastError();
   }
   template <bool DEV, bool GEN>
-  static void launch_x(tf_ctx& c, const LineK<LP>& L, const LP* ul, const LineK<LP>* Ld, cudaStream_t s) {
+  static cudaError_t launch_x(tf_ctx& c, const LineK<LP>& L, const LP* ul, const LineK<LP>* Ld, cudaStream_t s) {
     switch (c.nlx) {
       case 4: return narrow_x<4, DEV, GEN>(c, L, ul, Ld, s);
       case 8: return narrow_x<8, DEV, GEN>(c, L, ul, Ld, s);
       case 16: return narrow_x<16, DEV, GEN>(c, L, ul, Ld, s);
-      default:
-        if constexpr (kWide<GEN>)
-          k_xsweep<Mode, DEV, GEN><<<c.grid_x, kSweepThreads, smem_x, s>>>(c.mk, L, ul, (LP*)c.w, (LP*)c.fac_x,
-                                                                         c.px + c.n_rhs_parts, Ld, c.ahead);
     }
+    if constexpr (kWide<GEN>) {
+      if (c.nlx == 32) {
+        k_xsweep<Mode, DEV, GEN><<<c.grid_x, kSweepThreads, smem_x, s>>>(c.mk, L, ul, (LP*)c.w, (LP*)c.fac_x,
+                                                                       c.px + c.n_rhs_parts, Ld, c.ahead);
+        return cudaGetLastError();
+      }
+    }
+    return cudaErrorInvalidValue;
   }
   template <bool DEV, bool GEN>
-  static void launch_y(tf_ctx& c, const LineK<LP>& L, const double* u, const LP* ul, double* un, double* v,
+  static cudaError_t launch_y(tf_ctx& c, const LineK<LP>& L, const double* u, const LP* ul, double* un, double* v,
                        const LineK<LP>* Ld, const double* const* uio, cudaStream_t s) {
     switch (c.nly) {
       case 4: return narrow_y<4, DEV, GEN>(c, L, u, ul, un, v, Ld, uio, s);
       case 8: return narrow_y<8, DEV, GEN>(c, L, u, ul, un, v, Ld, uio, s);
       case 16: return narrow_y<16, DEV, GEN>(c, L, u, ul, un, v, Ld, uio, s);
-      default:
-        if constexpr (kWide<GEN>)
-          k_ysweep<Mode, DEV, GEN><<<c.grid_y, kSweepThreads, smem_y, s>>>(c.mk, L, u, ul, (const LP*)c.w, (LP*)c.fac_y,
-                                                                         un, v, c.py, Ld, uio, c.ahead);
     }
+    if constexpr (kWide<GEN>) {
+      if (c.nly == 32) {
+        k_ysweep<Mode, DEV, GEN><<<c.grid_y, kSweepThreads, smem_y, s>>>(c.mk, L, u, ul, (const LP*)c.w, (LP*)c.fac_y,
+                                                                       un, v, c.py, Ld, uio, c.ahead);
+        return cudaGetLastError();
+      }
+    }
+    return cudaErrorInvalidValue;
   }
   // Dynamic shared memory of a sweep kernel; two blocks share an SM only with
   // the largest shared carveout.
@@ -84,7 +95,12 @@ template <class Mode> struct Launch {
     return e ? e : allow(k_narrow_sweep<Mode, NL, 1, DEV, GEN>, smem_n<NL, 1>);
   }
   template <bool DEV, bool GEN> static cudaError_t prepare_narrow_nl(int nl) {
-    return nl == 4 ? prepare_narrow<4, DEV, GEN>() : (nl == 8 ? prepare_narrow<8, DEV, GEN>() : prepare_narrow<16, DEV, GEN>());
+    switch (nl) {
+      case 4: return prepare_narrow<4, DEV, GEN>();
+      case 8: return prepare_narrow<8, DEV, GEN>();
+      case 16: return prepare_narrow<16, DEV, GEN>();
+    }
+    return cudaErrorInvalidValue;
   }
   template <int NL> static cudaError_t prepare_solve_t() {
     cudaError_t e = allow(k_narrow_sweep<Mode, NL, 0, false, false, true>, smem_n<NL, 0>);
@@ -239,11 +255,8 @@ template <class Mode> struct Launch {
       if (c.part) return part::xsweep(c, dt);
     }
     const LineK<LP> L = line_consts<LP>(c.mk, step(c, dt));
-    if (power32(c))
-      launch_x<false, false>(c, L, film_lp(c, u_k), nullptr, c.stream);
-    else
-      launch_x<false, true>(c, L, film_lp(c, u_k), nullptr, c.stream);
-    return cudaGetLastError();
+    return power32(c) ? launch_x<false, false>(c, L, film_lp(c, u_k), nullptr, c.stream)
+                      : launch_x<false, true>(c, L, film_lp(c, u_k), nullptr, c.stream);
   }
   static cudaError_t ysweep_c(tf_ctx& c, const double* u_k, double dt, double* u_next,
                               double* v_out) {
@@ -251,11 +264,8 @@ template <class Mode> struct Launch {
       if (c.part) return part::ysweep(c, u_k, dt, u_next, v_out);
     }
     const LineK<LP> L = line_consts<LP>(c.mk, step(c, dt));
-    if (power32(c))
-      launch_y<false, false>(c, L, u_k, film_lp(c, u_k), u_next, v_out, nullptr, nullptr, c.stream);
-    else
-      launch_y<false, true>(c, L, u_k, film_lp(c, u_k), u_next, v_out, nullptr, nullptr, c.stream);
-    return cudaGetLastError();
+    return power32(c) ? launch_y<false, false>(c, L, u_k, film_lp(c, u_k), u_next, v_out, nullptr, nullptr, c.stream)
+                      : launch_y<false, true>(c, L, u_k, film_lp(c, u_k), u_next, v_out, nullptr, nullptr, c.stream);
   }
   // The whole run of an ensemble film as one graph (FP32-bulk, (3, 2) power
   // law, twisted sweeps): k_ens_begin, then WHILE (attempts) { explicit part
@@ -289,8 +299,8 @@ template <class Mode> struct Launch {
       };
       // one Newton iteration's sweeps and reductions
       auto sweeps = [&]() {
-        launch_x<true, false>(c, l0, (const LP*)c.ulp, &e->line, s);
-        launch_y<true, false>(c, l0, nullptr, (const LP*)c.ulp, nullptr, nullptr, &e->line, &e->p.uk, s);
+        if ((err = launch_x<true, false>(c, l0, (const LP*)c.ulp, &e->line, s))) return;
+        if ((err = launch_y<true, false>(c, l0, nullptr, (const LP*)c.ulp, nullptr, nullptr, &e->line, &e->p.uk, s))) return;
         k_ens_iter<<<1, 256, 0, s>>>(c.px, c.n_rhs_parts + c.grid_x, c.py, c.grid_y, e, hi);
       };
       if ((err = cudaGraphCreate(&g, 0))) return fail(err);
@@ -314,6 +324,7 @@ template <class Mode> struct Launch {
       k_rhs_strip<kRhsBoth, true><<<c.grid_pkx, kST, 0, s>>>(c.mk, rk0, nullptr, (HP*)c.bn, (LP*)c.w, (LP*)c.ulp, c.px,
                                                              c.strip_n, c.strip_rows, &e->rk_both, &e->p.cur);
       sweeps();
+      if (err) return fail(err);
       if ((err = cudaStreamEndCapture(s, &B))) return fail(err);
       {  // the last node of the chain: the one no other node depends on
         size_t nn = 0, ne = 0;
@@ -338,6 +349,7 @@ template <class Mode> struct Launch {
       k_rhs_strip<kRhsResidual, true><<<c.grid_pkx, kST, 0, s>>>(c.mk, rk0, nullptr, (HP*)c.bn, (LP*)c.w, (LP*)c.ulp,
                                                                  c.px, c.strip_n, c.strip_rows, &e->rk_res, &e->p.uk);
       sweeps();
+      if (err) return fail(err);
       if ((err = cudaStreamEndCapture(s, &I))) return fail(err);
       // end of the attempt: the result into nxt, its statistics, the controller
       if ((err = cudaStreamBeginCaptureToGraph(s, B, &ni, nullptr, 1, md))) return fail(err);

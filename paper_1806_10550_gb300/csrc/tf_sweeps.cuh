@@ -60,7 +60,7 @@ template <class HP, int T> struct RhsSmem {
 // first iteration (u_0 = u^n) from the stored b^n, as kRhsResidual would
 // form it (gscale the explicit part's, gscale2 the residual's).
 // T: the tile, 32 x 32, or 16 x 16 for films that it leaves SMs idle on (a
-// block's tile is a chain of FP64-bound stages; see set_shapes in tf_api.cu).
+// block's tile is a chain of FP64-bound stages; see tf_init in tf_api.cu).
 template <class Mode, int KIND, int T>
 __global__ void __launch_bounds__(256, 4)  // shared memory allows 4 blocks per SM: up to 64 registers
     k_rhs(ModelK M, RhsK<typename Mode::HP> RK, const double* __restrict__ u,
