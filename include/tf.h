@@ -250,10 +250,10 @@ int tf_advance(tf_ctx* ctx, double* h, double t0, double t_end, double dt0,
  *     set (their thread 0 runs tf_advance's decisions on the reduced
  *     scalars), with the film's Δt and Newton state in device memory.  The host waits once per film per
  *     call.  The block shapes of a film's kernels go by the lines that the
- *     films of a call have together (up to 1216, 2432, 12160, and more); its
- *     graph is built on the context's first such call of each size (0.13 ms
- *     for 200 x 170 cells) and kept.  Those first calls should come before
- *     any stream capture.
+ *     films of a call have together (one film; up to 1216, 2432, 12160, and
+ *     more); its graph is built on the context's first such call of each size
+ *     (0.13 ms for 200 x 170 cells) and kept.  Those first calls should come
+ *     before any stream capture.
  *     With timing enabled only tf_timing.launches is counted for these
  *     films.
  *   host engine (TF_ENSEMBLE_HOST, and every other context): the state

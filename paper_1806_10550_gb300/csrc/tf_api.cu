@@ -390,8 +390,10 @@ int sweep_lines(int n, int precision, bool general) {
 // counts: smaller blocks do more work per line, which only pays while the
 // films together leave SMs idle.  Whole runs in FP32-bulk, us at 8, 16 and 32
 // lines: 15 films of 4630 lines in all 1179, 1169, 1260; 11 of 7968 4365, 3536,
-// 3618; 23 of 10686 4583, 3787, 3936; 24 of 15365 7107, 5738, 5391.
-int shared_lines(long long lines) {
+// 3618; 23 of 10686 4583, 3787, 3936; 24 of 15365 7107, 5738, 5391.  A single
+// film is a film alone (16384 x 8, ten iterations: 4.6 ms, 10.2 in blocks of 32).
+int shared_lines(int films, long long lines) {
+  if (films < 2) return 0;
   return lines <= 8 * kSMs ? 4 : (lines <= 16 * kSMs ? 8 : (lines <= 80 * kSMs ? 16 : 32));
 }
 // The sweeps' block shape, at least `least` lines per block, and the residual's
@@ -428,7 +430,7 @@ struct SharedLines {
   SharedLines(int n_, tf_ctx* const* c) : n(n_), ctx(c) {
     long long lines = 0;
     for (int i = 0; i < n; ++i) lines += ctx[i]->p.nx > ctx[i]->p.ny ? ctx[i]->p.nx : ctx[i]->p.ny;
-    for (int i = 0; i < n; ++i) set_shapes(*ctx[i], shared_lines(lines));
+    for (int i = 0; i < n; ++i) set_shapes(*ctx[i], shared_lines(n, lines));
   }
   ~SharedLines() {
     for (int i = 0; i < n; ++i) set_shapes(*ctx[i], 0);
@@ -1028,7 +1030,7 @@ int tf_tune_line_solver(const tf_params* p, void* stream, const double* h, doubl
         break;
       }
       rc = tf_init(&q, st[(size_t)k], &ctx[(size_t)k]);
-      if (!rc) set_shapes(*ctx[(size_t)k], shared_lines((long long)copies * (q.nx > q.ny ? q.nx : q.ny)));
+      if (!rc) set_shapes(*ctx[(size_t)k], shared_lines(copies, (long long)copies * (q.nx > q.ny ? q.nx : q.ny)));
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!rc && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) rc = TF_ERR_CUDA;

@@ -30,9 +30,9 @@ struct ReportParts {
 };
 
 // A film's run as an instantiated graph, and the lines per sweep block and rows
-// per strip segment it was built with.  A context takes one of four shapes by
-// the lines that advance at once (shared_lines in tf_api.cu).
-constexpr int kEnsGraphs = 4;
+// per strip segment it was built with.  A context takes one of five shapes by
+// the films and lines that advance at once (shared_lines in tf_api.cu).
+constexpr int kEnsGraphs = 5;
 struct EnsGraph {
   cudaGraphExec_t exec;
   int nlx, nly, rows;

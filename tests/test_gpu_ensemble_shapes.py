@@ -81,3 +81,31 @@ def test_results_do_not_depend_on_the_set(torch):
         assert torch.equal(grids[0], ref)
     for c in ctxs + [single]:
         c.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(16384, 8), (8, 16384)])
+def test_one_film_is_a_film_alone(torch, nx, ny):
+    """A call with one film, and the tuner with one copy, run in the block
+    shapes of tf_advance: a long film's sweeps take half as long there as in the
+    blocks of many films.  The least of ten times of each within 30% of
+    tf_advance's (an iteration of the tuner also waits for the host: 50 us)."""
+    K = 10
+    p = tf.tf_params_default(nx=nx, ny=ny, ds=3.9, kappa=KAPPA, precision=tf.TF_FP32_BULK, newton_fixed_iter=K)
+    h = torch.from_numpy(S.spinodal_film(nx, ny, 1.0, 0.01, seed=6)).cuda()
+    ctx = tf.Context(p, stream=torch.cuda.Stream())
+    torch.cuda.synchronize()
+
+    def least(f):
+        best = float("inf")
+        for _ in range(11):
+            t = time.perf_counter()
+            f()
+            best = min(best, time.perf_counter() - t)
+        return best * 1e3
+
+    advance = least(lambda: tf.tf_advance(ctx, h, 0.0, 1e30, 1e-3, 1))
+    ensemble = least(lambda: tf.tf_ensemble_advance([ctx], [h], 0.0, 1e30, 1e-3, 1))
+    tuner = min(tf.tf_tune_line_solver(p, h, 1e-3, iters=K)["ms"][0] for _ in range(3))
+    assert ensemble <= 1.3 * advance, (ensemble, advance)
+    assert tuner <= 1.3 * advance / K + 0.05, (tuner, advance / K)
+    ctx.close()
