@@ -117,3 +117,23 @@ def test_films_at_an_8_byte_address(torch, mode, nx, ny):
     for a, b in zip(got[0][3:], got[1][3:]):
         assert torch.equal(a, b)
     ctx.close()
+
+
+def test_sweeps_of_general_exponents_cost_what_the_other_models_do(torch):
+    """4096^2 in FP32-bulk: an x sweep of (n, m) = (4, 3), whose mobilities are a
+    few products, takes less than 1.3 times one of the NLC model with its tanh
+    and reciprocals (least of five each)."""
+    n, best = 4096, {}
+    for which in ("nlc", "power43"):
+        _, p, h0, wm = setup(which, n, n, tf.TF_FP32_BULK)
+        p.newton_fixed_iter = 2
+        h = h0 * (1.0 + 0.01 * torch.rand((n, n), dtype=torch.float64, device="cuda"))
+        out = torch.empty_like(h)
+        ctx = tf.Context(p)
+        for _ in range(6):
+            tf.tf_timing_enable(ctx, True)
+            tf.tf_newton_adi_step(ctx, h, out, 1e-3 / wm)
+            t = tf.tf_timing_get(ctx)
+            best[which] = min(best.get(which, 1e30), t["x_ms"] / t["x_launches"])
+        ctx.close()
+    assert best["power43"] < 1.3 * best["nlc"], best
