@@ -427,10 +427,15 @@ void set_shapes(tf_ctx& c, int least) {
 struct SharedLines {
   int n;
   tf_ctx* const* ctx;
+  cudaError_t error = cudaSuccess;
   SharedLines(int n_, tf_ctx* const* c) : n(n_), ctx(c) {
     long long lines = 0;
     for (int i = 0; i < n; ++i) lines += ctx[i]->p.nx > ctx[i]->p.ny ? ctx[i]->p.nx : ctx[i]->p.ny;
-    for (int i = 0; i < n; ++i) set_shapes(*ctx[i], shared_lines(n, lines));
+    for (int i = 0; i < n; ++i) {
+      set_shapes(*ctx[i], shared_lines(n, lines));
+      const cudaError_t e = ctx[i]->ops->prepare_shapes(*ctx[i]);
+      if (e && !error) error = e;
+    }
   }
   ~SharedLines() {
     for (int i = 0; i < n; ++i) set_shapes(*ctx[i], 0);
@@ -912,6 +917,7 @@ int tf_ensemble_advance(int n, tf_ctx* const* ctx, double* const* h, const doubl
       if (ctx[j] == ctx[i]) return TF_ERR_ARG;  // one context per film
   }
   const SharedLines shapes(n, ctx);
+  TF_CK(shapes.error);
   // films on the graph engine: launched first, collected at the end
   std::vector<char> on_graph((size_t)n, 0);
   for (int i = 0; i < n; ++i) {
@@ -1030,7 +1036,10 @@ int tf_tune_line_solver(const tf_params* p, void* stream, const double* h, doubl
         break;
       }
       rc = tf_init(&q, st[(size_t)k], &ctx[(size_t)k]);
-      if (!rc) set_shapes(*ctx[(size_t)k], shared_lines(copies, (long long)copies * (q.nx > q.ny ? q.nx : q.ny)));
+      if (!rc) {
+        set_shapes(*ctx[(size_t)k], shared_lines(copies, (long long)copies * (q.nx > q.ny ? q.nx : q.ny)));
+        if (ctx[(size_t)k]->ops->prepare_shapes(*ctx[(size_t)k]) != cudaSuccess) rc = TF_ERR_CUDA;
+      }
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!rc && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) rc = TF_ERR_CUDA;

@@ -41,6 +41,7 @@ struct EnsGraph {
 struct Ops {
   size_t hp_bytes, lp_bytes;
   cudaError_t (*prepare)(tf_ctx& c);
+  cudaError_t (*prepare_shapes)(tf_ctx& c);  // after a change of nlx, nly
   cudaError_t (*explicit_part)(tf_ctx& c, const double* u_old, double dt);
   // explicit part plus the first iteration's right side (u_0 = u_old)
   cudaError_t (*explicit_rhs0)(tf_ctx& c, const double* u_old, double dt);
@@ -121,6 +122,7 @@ struct tf_ctx {
   cudaStream_t stream;
   size_t N;
   int nlx, nly;    // lines per block of the x and y sweeps
+  unsigned prepared;  // block shapes whose kernels are set up: nlx | nly << 8 of each
   int grid_x;      // blocks of the x sweep (nlx rows each)
   int grid_y;      // blocks of the y sweep (nly columns each)
   int rhs_tile, grid_rx, grid_ry;  // 2-D residual grid (16 x 16 or 32 x 32 tiles)

@@ -90,31 +90,28 @@ template <class Mode> struct Launch {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     return e ? e : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
   }
-  template <int NL, bool DEV, bool GEN> static cudaError_t prepare_narrow() {
-    cudaError_t e = allow(k_narrow_sweep<Mode, NL, 0, DEV, GEN>, smem_n<NL, 0>);
-    return e ? e : allow(k_narrow_sweep<Mode, NL, 1, DEV, GEN>, smem_n<NL, 1>);
-  }
-  template <bool DEV, bool GEN> static cudaError_t prepare_narrow_nl(int nl) {
+  template <int DIR, bool DEV, bool GEN> static cudaError_t prepare_sweep(int nl) {
     switch (nl) {
-      case 4: return prepare_narrow<4, DEV, GEN>();
-      case 8: return prepare_narrow<8, DEV, GEN>();
-      case 16: return prepare_narrow<16, DEV, GEN>();
+      case 4: return allow(k_narrow_sweep<Mode, 4, DIR, DEV, GEN>, smem_n<4, DIR>);
+      case 8: return allow(k_narrow_sweep<Mode, 8, DIR, DEV, GEN>, smem_n<8, DIR>);
+      case 16: return allow(k_narrow_sweep<Mode, 16, DIR, DEV, GEN>, smem_n<16, DIR>);
+    }
+    if constexpr (kWide<GEN>) {
+      if (nl == 32) {
+        if constexpr (DIR == 0) return allow(k_xsweep<Mode, DEV, GEN>, smem_x);
+        else return allow(k_ysweep<Mode, DEV, GEN>, smem_y);
+      }
     }
     return cudaErrorInvalidValue;
+  }
+  template <bool DEV, bool GEN> static cudaError_t prepare_sweeps(const tf_ctx& c) {
+    const cudaError_t e = prepare_sweep<0, DEV, GEN>(c.nlx);
+    return e ? e : prepare_sweep<1, DEV, GEN>(c.nly);
   }
   template <int NL> static cudaError_t prepare_solve_t() {
     cudaError_t e = allow(k_narrow_sweep<Mode, NL, 0, false, false, true>, smem_n<NL, 0>);
     return e ? e : allow(k_narrow_sweep<Mode, NL, 1, false, false, true>, smem_n<NL, 1>);
   }
-  template <bool DEV, bool GEN> static cudaError_t prepare_sweeps() {
-    cudaError_t e;
-    if constexpr (kWide<GEN>) {
-      if ((e = allow(k_xsweep<Mode, DEV, GEN>, smem_x)) || (e = allow(k_ysweep<Mode, DEV, GEN>, smem_y))) return e;
-    }
-    if ((e = prepare_narrow<4, DEV, GEN>()) || (e = prepare_narrow<8, DEV, GEN>())) return e;
-    return prepare_narrow<16, DEV, GEN>();
-  }
-
   static StepK step(const tf_ctx& c, double dt) {
     StepK k;
     k.theta_dt = c.p.theta * dt;
@@ -122,9 +119,9 @@ template <class Mode> struct Launch {
     return k;
   }
 
-  // The attributes of the kernels that a context runs (an attribute call a
-  // kernel takes about a microsecond; the ensemble graphs' and the transposed
-  // solves' are set on their first use).
+  // The attributes of the kernels that a context runs (a kernel's take about a
+  // microsecond; the ensemble graphs' and the transposed solves' are set on
+  // their first use).
   static cudaError_t prepare(tf_ctx& c) {
     cudaError_t e;
     if (!c.packed_rhs &&
@@ -132,12 +129,19 @@ template <class Mode> struct Launch {
       return e;
     if constexpr (kF32B) {
       if (c.part) return part::prepare();
-      if (!power32(c)) {  // one shape whatever runs beside the film (set_shapes)
-        e = prepare_narrow_nl<false, true>(c.nlx);
-        return e || c.nly == c.nlx ? e : prepare_narrow_nl<false, true>(c.nly);
-      }
     }
-    return power32(c) ? prepare_sweeps<false, false>() : prepare_sweeps<false, true>();
+    return prepare_shapes(c);
+  }
+  // Those of the sweeps in the context's present block shapes, once per shape: a
+  // film alone runs in one, and setting up all of them added 8 us to a context's
+  // creation (64^2, FP64: 233 us without, 241 with).
+  static cudaError_t prepare_shapes(tf_ctx& c) {
+    if (c.part) return cudaSuccess;
+    const unsigned need = (unsigned)(c.nlx | c.nly << 8);  // 4, 8, 16 or 32 each: a bit
+    if ((c.prepared & need) == need) return cudaSuccess;
+    const cudaError_t e = power32(c) ? prepare_sweeps<false, false>(c) : prepare_sweeps<false, true>(c);
+    if (!e) c.prepared |= need;
+    return e;
   }
 
   static cudaError_t explicit_part_c(tf_ctx& c, const double* u_old, double dt) {
@@ -282,7 +286,7 @@ template <class Mode> struct Launch {
       if (!c.packed_rhs || c.part) return cudaErrorNotSupported;
       cudaStream_t s = nullptr;
       cudaGraph_t g = nullptr, B = nullptr, I = nullptr;
-      cudaError_t err = prepare_sweeps<true, false>();
+      cudaError_t err = prepare_sweeps<true, false>(c);
       if (err) return err;
       err = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
       if (err) return err;
@@ -379,6 +383,7 @@ template <class Mode> Ops make_ops() {
   o.hp_bytes = sizeof(typename Mode::HP);
   o.lp_bytes = sizeof(typename Mode::LP);
   o.prepare = &L::prepare;
+  o.prepare_shapes = &L::prepare_shapes;
   o.explicit_part = &L::explicit_part_c;
   o.explicit_rhs0 = &L::explicit_rhs0_c;
   o.report = &L::report_c;
