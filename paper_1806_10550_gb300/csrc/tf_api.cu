@@ -397,10 +397,13 @@ int shared_lines(int films, long long lines) {
   return lines <= 8 * kSMs ? 4 : (lines <= 16 * kSMs ? 8 : (lines <= 80 * kSMs ? 16 : 32));
 }
 // The sweeps' block shape, at least `least` lines per block, and the residual's
-// strips.  In FP32-bulk with the out-of-line mobility models the sweeps' shapes
-// round differently, so there the shape depends on the film alone.
+// strips.  Every shape rounds alike.  In FP32-bulk the general models have no
+// blocks of 32: films at once, us with (4, 3) at 4, 8, 16 and 32 lines: 24 of
+// 1024^2 28350, 22909, 15811, 14333; 32 of 512^2 11320, 9016, 6864, 7841; 64 of
+// 256^2 8387, 7657, 7383, 9484; NLC 49975, 42920, 36913, 35243; 17323, 14919,
+// 13415, 13132; 11654, 11055, 10919, 11992.
 void set_shapes(tf_ctx& c, int least) {
-  if (c.p.precision != TF_FP64 && !c.packed_rhs) least = 0;
+  if (c.p.precision != TF_FP64 && !c.packed_rhs && least > 16) least = 16;
   const bool general = !(c.mk.model == TF_MODEL_POWERLAW && c.mk.n == 3 && c.mk.m == 2);
   const int x = sweep_lines(c.p.ny, c.p.precision, general), y = sweep_lines(c.p.nx, c.p.precision, general);
   c.nlx = x > least ? x : least;

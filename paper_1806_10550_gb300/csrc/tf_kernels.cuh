@@ -217,7 +217,6 @@ template <class T> TF_HD MobC<T> mob_consts(const ModelK& M) {
 // or recompute them per cell.
 template <class T> struct LineK {
   MobC<T> ml;
-  T inv_ds2;  // 1/ds^2
   T k3, k1;   // theta dt/(2 ds^4) and theta dt/(2 ds^2): the band's face scales
   // folded factors of the (n, m) = (3, 2) power law (ml.pl32):
   // F0 = k3 C h^3, F1 = k1 A1 - k1 B1 / h, D0 = (k1 / ds^2) 3 C h^2 (the
@@ -227,7 +226,6 @@ template <class T> struct LineK {
 template <class T> TF_HD LineK<T> line_consts(const ModelK& M, const StepK& K) {
   LineK<T> L;
   L.ml = mob_consts<T>(M);
-  L.inv_ds2 = (T)M.inv_ds2;
   const double k3 = 0.5 * K.theta_dt * M.inv_ds3 * M.inv_ds, k1 = 0.5 * K.theta_dt * M.inv_ds2;
   L.k3 = (T)k3;
   L.k1 = (T)k1;

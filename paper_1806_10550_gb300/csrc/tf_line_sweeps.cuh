@@ -147,7 +147,7 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 
 // Per-cell film values, pre-scaled for the band: with k3 = theta dt/(2 ds^4)
 // and k1 = theta dt/(2 ds^2),
-//   F0 = k3 f0, F1 = k1 f1, D0 = k1 f0', D1 = k1 f1',
+//   F0 = k3 f0, F1 = k1 f1, D0 = k3 f0' (lap unscaled), D1 = k1 f1',
 // so that for the face between line cells p and q (the scaled dF of
 // face_dF): c3 = F0_p + F0_q, Bd = F1_p + F1_q,
 //   t_p = D0_p (lap_q - lap_p) + D1_p (u_q - u_p), t_q likewise, and
@@ -156,34 +156,35 @@ template <class LP> struct CellS {
   LP u, lap, F0, F1, D0, D1;
 };
 
-// uc: the cell's height; lap: its unscaled Laplacian.
+// uc: the cell's height; lap: its Laplacian, left unscaled: its 1/ds^2 makes
+// k1 into k3 in D0.  F0 and F1 are rounded as products of their own (never fused
+// into the face sums), so that every instantiation of the sweeps rounds the band
+// alike, whatever films run beside it.
 template <class LP>
-__device__ __forceinline__ CellS<LP> cell_scaled(const MobC<LP>& ml, LP inv_ds2, LP k3, LP k1, LP uc, LP lap) {
+__device__ __forceinline__ CellS<LP> cell_scaled(const MobC<LP>& ml, LP k3, LP k1, LP uc, LP lap) {
   CellS<LP> X;
   X.u = uc;
-  X.lap = lap * inv_ds2;
+  X.lap = lap;
   const LP s = rcp3(uc);
   LP f0, f1, d0, d1;
   mobility_all(ml, uc, s, f0, f1, d0, d1);
-  X.F0 = k3 * f0;
-  X.F1 = k1 * f1;
-  X.D0 = k1 * d0;
+  X.F0 = mul_rn(k3, f0);
+  X.F1 = mul_rn(k1, f1);
+  X.D0 = k3 * d0;
   X.D1 = k1 * d1;
   return X;
 }
 
 // The same values for the (n, m) = (3, 2) power law with the constant
-// factors folded on the host (LineK): the Laplacian is left unscaled and
-// 1/ds^2 moves into D0, so faces see the same products.
+// factors folded on the host (LineK).
 template <class LP>
 __device__ __forceinline__ CellS<LP> cell_pl32(const LineK<LP>& L, LP uc, LP lap) {
   CellS<LP> X;
   X.u = uc;
   X.lap = lap;
   const LP s = rcp3(uc), h2 = uc * uc;
-  // F0 rounded as a product of its own (never fused into the face sums
-  // F0_p + F0_q) and F1 as one written-out fma: every instantiation of the
-  // sweeps then rounds the band alike
+  // F0 rounded as a product of its own and F1 as one written-out fma, as in
+  // cell_scaled
   X.F0 = mul_rn(L.pF0, h2 * uc);
   X.F1 = fma(-L.pF1b, s, L.pF1a);
   X.D0 = L.pD0 * h2;
@@ -244,7 +245,7 @@ __device__ __forceinline__ void band_rows(const LineK<LP>& L, Acc A, int ia, int
     if constexpr (PL32)
       C[s + 1] = cell_pl32<LP>(L, uc, lap);
     else
-      C[s + 1] = cell_scaled<LP>(L.ml, L.inv_ds2, L.k3, L.k1, uc, lap);
+      C[s + 1] = cell_scaled<LP>(L.ml, L.k3, L.k1, uc, lap);
   }
   LP F[G + 1][4];
 #pragma unroll
