@@ -747,11 +747,21 @@ ADJOINT_METRIC = ("adjoint film cell-steps/s: gradient of |h(T) - h_target|^2 ov
 
 # Algorithmic bytes per cell of one launch of each adjoint kernel group:
 # the transposed solve reads the five band diagonals and the right side and
-# writes the solution (56 B); a line derivative reads u_k, w, lambda and
-# updates the cotangent (40 B); the D derivative the same without w (32 B).
-# The per-iterate tables, the elimination scratch and the Laplacian
-# cotangent pass are implementation traffic.
-ADJ_BYTES_PER_CELL = {"solve_t": 56.0, "line_x": 40.0, "line_y": 40.0, "D": 32.0}
+# writes the solution (56 B); an iteration's derivatives (of both lines and of
+# D, one pass, in the group line_x) read u_k, w_k, v_k and both lines' lambda and
+# update the cotangents of u_k and b (72 B); the explicit part's D derivative
+# reads u and the cotangent of b and updates that of u (32 B).  The per-iterate
+# tables, the elimination scratch and the Laplacian cotangent pass are
+# implementation traffic.
+ADJ_BYTES_PER_CELL = {"solve_t": 56.0, "line_x": 72.0, "D": 32.0}
+
+
+def adjoint_reverse_launches(K, ns):
+    """Launches of the reverse over ns steps of K iterations: those of each
+    timed group's dominant kernel, and all of them (per iteration the tables, two
+    bands, two solves, the derivatives and the Laplacian's transpose; per step an
+    axpy, the D derivative and the Laplacian's transpose)."""
+    return {"solve_t": 2 * K * ns, "line_x": K * ns, "D": ns}, ns * (7 * K + 3)
 
 
 def adjoint_config(w, world):
@@ -851,7 +861,7 @@ def run_adjoint(args, w):
     # (the tape's timing, from the timed region)
     per = {k: v / S_ for k, v in groups.items()}
     fwd = kernel_table(dict(timing=tim), N, 8)
-    rev_launches = {"solve_t": 2 * K * ns, "line_x": K * ns, "line_y": K * ns, "D": (K + 1) * ns}
+    rev_launches, rev_total = adjoint_reverse_launches(K, ns)
     cand = {k: (n_, ms_, b) for k, (n_, ms_, b) in fwd.items()}
     cand.update({k: (rev_launches[k], per[k], ADJ_BYTES_PER_CELL[k] * N * N) for k in rev_launches})
     dom = max(cand, key=lambda k: cand[k][1])
@@ -869,11 +879,9 @@ def run_adjoint(args, w):
         data="synthetic", config=adjoint_config(w, world), g_theta=r["g_theta"], g_kappa=r["g_kappa"],
         checkpoints=dict(every=tinfo["every"], count=tinfo["checkpoints"], tape_bytes=tinfo["bytes"]),
         group_ms_per_step={k: round(v, 1) for k, v in per.items()}, roofline=roof,
-        # the forward kernels as the context counts them in one gradient;
-        # the reverse per step and iteration 1 tables, 2 band, 2 solve, 2
-        # line and 1 D derivative, 3 Laplacian-transpose and 2 axpy kernels,
-        # then 1 axpy, 1 D derivative and 1 Laplacian-transpose
-        gpu_launches=S_ * (tim["launches"] + ns * (13 * K + 3)),
+        # the forward kernels as the context counts them in one gradient, and
+        # the reverse's
+        gpu_launches=S_ * (tim["launches"] + rev_total),
         e2e=dict(value=job_rate(dist, N * N * ns * S_, ms_e2e), unit="cell-steps/s",
                  h2d_bytes_per_step=N * N * 8, d2h_bytes_per_step=N * N * 8),
     )
