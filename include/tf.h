@@ -374,9 +374,12 @@ int tf_residual_noalloc(const tf_params* p, void* stream, const double* h_k,
  * g_h: device output grid (not aliasing h_old, g or h_new); g_kappa,
  * g_theta: host outputs or NULL (g_theta = g_kappa dkappa/dtheta_c when
  * kappa was derived from the contact angle, else 0).  K: 1..64.
- * Workspace (3K + 16 grids and the solves' factors, about 4 more) is allocated on first use and kept by the
- * context.  Synchronises the context's stream.  Returns TF_OK, TF_ERR_ARG,
- * TF_ERR_NOMEM or TF_ERR_CUDA (or a forward iteration's error).         */
+ * Workspace is allocated on first use and kept by the context: 3K + 16 grids,
+ * and the solves' factors, 3 doubles a cell of the lines of one direction
+ * (whichever needs more) with half a line rounded up to a multiple of 24 cells
+ * and the lines to a multiple of 16: 3.1 grids at 1024^2, more where lines are
+ * short (16 at 9 x 2434).  Synchronises the context's stream.  Returns TF_OK,
+ * TF_ERR_ARG, TF_ERR_NOMEM or TF_ERR_CUDA (or a forward iteration's error).  */
 int tf_adjoint_step(tf_ctx* ctx, const double* h_old, double dt, int K, const double* g,
                     double* h_new, double* g_h, double* g_kappa, double* g_theta);
 

@@ -124,12 +124,17 @@ TF_HD float rcp(float x) {
   return 1.0f / x;
 #endif
 }
-// Reciprocal of the FP64 line solves and of the FP64 Jacobian's heights: the
-// hardware's approximate reciprocal r0 (at least 2^-18 good: e = 1 - x r0) and
-// one third-order step, 1/x = r0 (1 + e + e^2) + O(e^3): three FP64 operations,
-// rounded once at the end.  What bounds the FP64 sweeps is the number of FP64
-// instructions (a warp's takes 65 cycles of its sub-partition's pipe whatever
-// its lanes).  Zero, non-finite and extreme arguments take the division.
+// Reciprocal of the FP64 kernels: heights (of the residual, the Jacobian and the
+// adjoint's tables), the NLC and polymer Pi', pivots, the Newton test.  The
+// hardware's approximate reciprocal r0, with e = 1 - x r0 at most 2^-19.9 (measured
+// over all 2^20 upper significands, which are all that it reads), and one step of
+// the cubically convergent iteration of M. Altman (Pacific J. Math. 10 (1960)
+// 1107), the geometric series cut after its third term: 1/x = r0 (1 + e + e^2) +
+// O(e^3).  Three FP64 operations, rounded once at the end: within one unit in the
+// last place of the division, and its own bits in 99.9% of arguments.  What bounds
+// the FP64 sweeps is the number of FP64 instructions (a warp's takes 65 cycles of
+// its sub-partition's pipe whatever its lanes).  Zero, non-finite and extreme
+// arguments take the division.
 __device__ __forceinline__ double rcp3(double x) {
   const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
   if (ex - 64u > 1918u) return 1.0 / x;  // r0 and 1/x are normal for exponents 64 .. 1982
