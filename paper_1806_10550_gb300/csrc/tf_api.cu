@@ -374,12 +374,16 @@ TuneKey tune_key(const tf_params& p) { return TuneKey{p.nx, p.ny, p.precision, p
 // / y sweep at 4, 8, 16 and 32 lines a block: FP32-bulk 512^2 22/27, 23/29, 27/35,
 // 38/45; 1024^2 39/47, 37/45, 45/57, 69/81; 2048^2 129/144, 74/90, 79/100, 130/154;
 // 4096^2 at 8, 16 and 32 lines 267/326, 182/235, 254/305; 8192^2 at 16 and 32
-// 627/791, 734/802.  With the out-of-line mobilities (NLC) the producers are
-// the longest role, and 4 lines win further: 1024^2 86/89, 115/121, 134/143;
-// 2048^2 309/322, 227/241, 255/270; 4096^2 at 8 and 16 lines 875/928, 644/665.
-// FP64 512^2 164/166, 170/174, 202/211, 331/351; 1024^2 377/615, 317/322, 379/391,
-// 647/687; 2048^2 at 8, 16 and 32 lines 1197/1221, 732/752, 1278/1348; from there
-// on one block an SM, and blocks of 32 do less work per line.
+// 627/791, 734/802.  With the general models' mobilities the producers are the
+// longest role, and 4 lines win further (at 4, 8 and 16 lines): NLC 1024^2 60/65,
+// 72/78, 81/87; 2048^2 211/222, 150/164, 151/160; 4096^2 at 8 and 16 561/606,
+// 362/388; 8192^2 at 16 and 32 1378/1507, 1315/1410; (4, 3) 1450/1484, 1289/1397.
+// FP64 512^2 164/166, 170/174, 202/211, 331/351; 1024^2 511/543, 289/294, 365/391,
+// 636/677; 2048^2 at 8, 16 and 32 lines 1078/1097, 698/747, 1255/1331; 4096^2 at 16
+// and 32 2735/2923, 2489/2636.  The general models rank their shapes the same way
+// in FP64: NLC 2048^2 2300/2302, 1819/1825, 3234/3301; 4096^2
+// 7211/7231, 6471/6587.  (Where blocks of 32 begin a second wave, 16 are faster
+// again: 6500^2 6472/6914, 7827/8307.)
 constexpr int kSMs = 152;
 int sweep_lines(int n, int precision, bool general) {
   if (n <= 4 * kSMs * (precision != TF_FP64 && general ? 2 : 1)) return 4;
