@@ -92,8 +92,8 @@ def current_counters(table, mode, root=CSRC) -> dict:
 # FP64 operations executed per cell by each FP64-mode kernel (DFMA counted
 # as 2, DADD and DMUL as 1), from an ncu capture of the FP64-mode kernels at
 # 4096^2 (per cell they do not depend on the grid size).
-FP64_FLOPS_PER_CELL = {"rhs": (46.14, "b7f77f9a109008d3"), "x_sweep": (85.91, "1453e94b4cd1b98b"),
-                       "y_sweep": (102.91, "1453e94b4cd1b98b")}
+FP64_FLOPS_PER_CELL = {"rhs": (41.62, "f2e6ffe6fd4d5c3a"), "x_sweep": (75.47, "c432a6afae8018b4"),
+                       "y_sweep": (84.47, "c432a6afae8018b4")}
 
 
 class ClockSampler:
@@ -293,8 +293,8 @@ def kernel_table(res, N, lp):
 # DRAM bytes (read + write) per cell per launch of each FP32-bulk kernel,
 # from an ncu capture of the FP32-bulk kernels at 4096^2 (traffic scales
 # with the cells).
-TRAFFIC_PER_CELL_F32B = {"rhs": (24.27, "7980ad0cf0226350"), "x_sweep": (31.23, "1453e94b4cd1b98b"),
-                         "y_sweep": (44.37, "1453e94b4cd1b98b"), "explicit": (21.68, "7980ad0cf0226350")}
+TRAFFIC_PER_CELL_F32B = {"rhs": (24.24, "6d31a1589dc33180"), "x_sweep": (31.91, "c432a6afae8018b4"),
+                         "y_sweep": (44.49, "c432a6afae8018b4"), "explicit": (21.66, "6d31a1589dc33180")}
 
 
 def ncu_counters_apply(w) -> bool:
