@@ -66,7 +66,9 @@ extern "C" {
 #define TF_FP32_BULK 1 /* residual, explicit part, update and norms in
                           double-float (FP32 pairs, >= 47-bit significand) on
                           the FP32 pipes; Jacobian assembly and pentadiagonal
-                          solves in FP32; state stays IEEE double           */
+                          solves in FP32; state stays IEEE double.  Floats
+                          carry the fluxes: use units of length in which
+                          heights and ds are near 1                         */
 
 /* line solvers of the pentadiagonal systems (eq. LUFactorization); both
    solve every line exactly, without pivoting                              */
